@@ -1,0 +1,74 @@
+#!/usr/bin/env python3
+"""Writes phi_table.h: piecewise polynomials of the two functions of z = delta / sigma
+that the FP64 pair arithmetic needs (pair_math64.cuh),
+  F(z) = phi(z) / Phi(z)   and   G(z) = log Phi(z),
+phi and Phi the standard normal density and distribution function, on the
+nodes c = i / 64, i = 0 .. 608 (z up to 9.5): degree 5 in t = z - c, |t| <= 1/128,
+each the polynomial that interpolates the function at the 6 Chebyshev points
+of its interval (computed with 40 digits, coefficients rounded to FP64).
+
+Usage: python gen_phi_table.py > phi_table.h
+"""
+from mpmath import cos, erfc, exp, log, mp, mpf, pi, sqrt
+
+mp.dps = 40
+PER_UNIT, NODES, DEG = 64, 609, 5
+HALF = mpf(1) / (2 * PER_UNIT)
+
+
+def cdf(z):
+    return erfc(-z / sqrt(2)) / 2
+
+
+def f(z):
+    return exp(-z * z / 2) / sqrt(2 * pi) / cdf(z)
+
+
+def g(z):
+    return log(cdf(z)) if z < 1 else log(1 - erfc(z / sqrt(2)) / 2)
+
+
+CHEB = [HALF * cos((2 * k + 1) * pi / (2 * (DEG + 1))) for k in range(DEG + 1)]
+
+
+def fit(fn, c):
+    """Monomial coefficients (in t) of the interpolant at the Chebyshev points: Newton's divided differences, expanded."""
+    d = [fn(c + t) for t in CHEB]
+    for k in range(1, DEG + 1):
+        for j in range(DEG, k - 1, -1):
+            d[j] = (d[j] - d[j - 1]) / (CHEB[j] - CHEB[j - k])
+    poly = [d[DEG]]
+    for k in range(DEG - 1, -1, -1):
+        shifted = [mpf(0)] + poly
+        poly = [a - CHEB[k] * b for a, b in zip(shifted, poly + [mpf(0)])]
+        poly[0] += d[k]
+    return poly
+
+
+def main():
+    worst = [mpf(0), mpf(0)]
+    rows = []
+    for i in range(NODES):
+        c = mpf(i) / PER_UNIT
+        row = []
+        for q, fn in enumerate((f, g)):
+            p = fit(fn, c)
+            for u in (-1, mpf(-7) / 10, mpf(-1) / 4, mpf(1) / 3, mpf(8) / 10, 1):
+                t = u * HALF
+                v = sum(a * t ** k for k, a in enumerate(p))
+                worst[q] = max(worst[q], abs(v - fn(c + t)))
+            row += [float(a) for a in reversed(p)]
+        rows.append(row)
+    print("// Generated by gen_phi_table.py -- do not edit.")
+    print("// Node i, t = z - i/64: F = phi/Phi and G = log Phi as degree-5 polynomials, highest power first;")
+    print("// largest absolute error before the coefficients' rounding: F %.1e, G %.1e." % (worst[0], worst[1]))
+    print("#pragma once")
+    print("constexpr int kPhiPerUnit = %d, kPhiNodes = %d, kPhiDeg = %d;" % (PER_UNIT, NODES, DEG))
+    print("__device__ const double g_phi_table[kPhiNodes * 2 * (kPhiDeg + 1)] = {")
+    for r in rows:
+        print(",".join("%.17g" % v for v in r) + ",")
+    print("};")
+
+
+if __name__ == "__main__":
+    main()

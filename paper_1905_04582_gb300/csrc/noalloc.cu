@@ -9,13 +9,17 @@
 // fixed file-scope array below, which every GPU that loads this library
 // holds until the process exits.
 //
-// Work split: one warp per row i of the full N x N matrix Y; the lanes stride
-// over j != i, so every pair is visited twice (once per end, as the per-row
-// gradient sums of the paper's Algorithm 2) and no column partials are
-// needed.  Arithmetic is FP64 (CUDA's sqrt / erfc / log1p / exp), the same
-// per-pair formulas as the FP64 path.  Each block writes its partial sums of
-// the scalar terms into the scratch array; a second, single-block kernel sums
-// them in a fixed order.
+// Work split: one CTA per row i of the full N x N matrix Y (several rows in
+// turn beyond N = 8192); its threads stride over j != i, so every pair is
+// visited twice (once per end, as the per-row gradient sums of the paper's
+// Algorithm 2) and no column partials are needed.  The per-pair arithmetic is
+// that of the FP64 path (pair_math64.cuh), bound by the FP64 pipe; log Phi
+// and the other scalar terms are evaluated only for j > i.  A whole CTA per
+// row rather than a warp: the rows then come in pieces small enough to end
+// together on 152 SMs, and the table that each CTA reads is loaded while the
+// CTAs beside it compute.  Each block writes its partial sums of the scalar
+// terms into the scratch array; a second, single-block kernel sums them in a
+// fixed order.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -25,12 +29,16 @@
 
 #include "mds.h"
 #include "mds_internal.h"
+#include "pair_math.cuh"
+#include "pair_math64.cuh"
 
+namespace mds {
 namespace {
 
-constexpr int kNaWarps = 8;                       // rows per block
+constexpr int kNaWarps = 4;
 constexpr int kNaThreads = 32 * kNaWarps;
-constexpr int kNaMaxBlocks = 8192;                // => N <= 65536
+constexpr int kNaMaxBlocks = 8192;
+constexpr int64_t kNaMaxN = 65536;
 constexpr int kNaParts = 4;                       // e^2, m*delta, log Phi, spare
 
 // The scratch: per-block partial sums, then the three final sums.
@@ -40,74 +48,88 @@ constexpr int kMaxDevices = 64;
 std::mutex g_na_mu;
 double *g_na_ptr[kMaxDevices] = {};
 
+// Row sums: gradient in units of -sigma^2 (see pair_f64_kernel), then the scalars.
 template <int D>
-__global__ void __launch_bounds__(kNaThreads) noalloc_rows_kernel(int64_t n, const float *y, int64_t ld,
-                                                                  const double *x, double sigma, double *grad,
-                                                                  double *part) {
-    constexpr double kInvSqrt2Pi = 0.39894228040143267794;
-    constexpr double kInvSqrt2 = 0.70710678118654752440;
-    __shared__ double red[kNaWarps][3];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t i = static_cast<int64_t>(blockIdx.x) * kNaWarps + warp;
-    const double inv_s = 1.0 / sigma, inv_s2 = inv_s * inv_s;
-    double g[D];
+struct RowSums {
+    double v[Pow2<D + 3>::value];
+};
+
+// Pairs (i, j) of row i for j in [lo, hi), a thread each in turn; SCALARS: their scalar terms too.
+template <int D, bool SCALARS>
+__device__ __forceinline__ void row_part(const double *tab, const Sigma64 &sg, const double (&xi)[D],
+                                         const double *x, const float *yrow, int64_t lo, int64_t hi, RowSums<D> &acc) {
+    for (int64_t j0 = lo; j0 < hi; j0 += kNaThreads) {
+        const bool in = j0 + threadIdx.x < hi;
+        const int64_t j = in ? j0 + threadIdx.x : lo;
+        double dl[D];
+        double d2 = 1e-300;  // see root64
 #pragma unroll
-    for (int k = 0; k < D; ++k) g[k] = 0.0;
-    double e2 = 0.0, md = 0.0, lp = 0.0;
-    if (i < n) {
+        for (int k = 0; k < D; ++k) {
+            dl[k] = xi[k] - x[j * D + k];
+            d2 = fma(dl[k], dl[k], d2);
+        }
+        double del, inv;
+        root64(d2, del, inv);
+        double w = in ? widen(yrow[j]) - del : 0.0;  // y - delta
+        if constexpr (SCALARS) acc.v[D] = fma(w, w, acc.v[D]);
+        const bool near = in && phi_near(sg, del);
+        if (__any_sync(0xffffffffu, near)) {
+            double F, G;
+            phi_eval<SCALARS>(tab, sg, del, F, G);
+            F = near ? F : 0.0;
+            if constexpr (SCALARS) {
+                acc.v[D + 1] = fma(F, del, acc.v[D + 1]);
+                acc.v[D + 2] += near ? G : 0.0;
+            }
+            w = fma(F, sg.neg_s, w);
+        }
+        w *= inv;
+#pragma unroll
+        for (int k = 0; k < D; ++k) acc.v[k] = fma(w, dl[k], acc.v[k]);
+    }
+}
+
+template <int D>
+__global__ void __launch_bounds__(kNaThreads, 3) noalloc_rows_kernel(int64_t n, int rows, const float *y, int64_t ld,
+                                                                     const double *x, double sigma, double *grad,
+                                                                     double *part) {
+    constexpr int V = D + 3, P = Pow2<V>::value;
+    extern __shared__ __align__(16) unsigned char na_smem[];
+    double *tab = reinterpret_cast<double *>(na_smem);
+    __shared__ double red[kNaWarps][V];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const Sigma64 sg = sigma64(sigma);
+    phi_table_load(tab);
+    __syncthreads();
+    double scalar = 0.0;  // threads D .. D + 2: the block's sums of the scalar terms
+    const int64_t i1 = min(n, static_cast<int64_t>(blockIdx.x + 1) * rows);
+    for (int64_t i = static_cast<int64_t>(blockIdx.x) * rows; i < i1; ++i) {
+        RowSums<D> acc;
+#pragma unroll
+        for (int q = 0; q < P; ++q) acc.v[q] = 0.0;
         double xi[D];
 #pragma unroll
         for (int k = 0; k < D; ++k) xi[k] = x[i * D + k];
         const float *yrow = y + i * ld;
-        for (int64_t j = lane; j < n; j += 32) {
-            if (j == i) continue;
-            double dl[D];
-            double d2 = 0.0;
+        row_part<D, false>(tab, sg, xi, x, yrow, 0, i, acc);
+        row_part<D, true>(tab, sg, xi, x, yrow, i + 1, n, acc);
+        lane_reduce<P, 5>(acc.v, lane, 0);
+        bool writer;
+        const int base = reduced_base<P, 5>(lane, 0, writer);
+        if (writer && base < V) red[warp][base] = acc.v[0];
+        __syncthreads();
+        if (tid < V) {
+            double v = red[0][tid];
 #pragma unroll
-            for (int k = 0; k < D; ++k) {
-                dl[k] = xi[k] - x[j * D + k];
-                d2 = fma(dl[k], dl[k], d2);
-            }
-            const double del = sqrt(d2);
-            const double inv = del > 0.0 ? 1.0 / del : 0.0;
-            const double e = static_cast<double>(yrow[j]) - del;
-            const double z = del * inv_s;
-            const double qz = 0.5 * erfc(z * kInvSqrt2);
-            const double m = exp(-0.5 * z * z) * kInvSqrt2Pi / (1.0 - qz);
-            const double wi = (m * inv_s - e * inv_s2) * inv;
-#pragma unroll
-            for (int k = 0; k < D; ++k) g[k] -= wi * dl[k];
-            if (j > i) {  // scalar terms once per pair
-                e2 = fma(e, e, e2);
-                md = fma(m, del, md);
-                lp += log1p(-qz);
-            }
+            for (int w = 1; w < kNaWarps; ++w) v += red[w][tid];
+            if (tid < D)
+                grad[i * D + tid] = sg.inv_s * sg.inv_s * v;
+            else
+                scalar += v;
         }
+        __syncthreads();  // red is free for the next row
     }
-#pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) {
-#pragma unroll
-        for (int k = 0; k < D; ++k) g[k] += __shfl_xor_sync(0xffffffffu, g[k], o);
-        e2 += __shfl_xor_sync(0xffffffffu, e2, o);
-        md += __shfl_xor_sync(0xffffffffu, md, o);
-        lp += __shfl_xor_sync(0xffffffffu, lp, o);
-    }
-    if (lane == 0) {
-        if (i < n) {
-#pragma unroll
-            for (int k = 0; k < D; ++k) grad[i * D + k] = g[k];
-        }
-        red[warp][0] = e2;
-        red[warp][1] = md;
-        red[warp][2] = lp;
-    }
-    __syncthreads();
-    if (threadIdx.x < 3) {
-        double v = red[0][threadIdx.x];
-#pragma unroll
-        for (int w = 1; w < kNaWarps; ++w) v += red[w][threadIdx.x];
-        part[blockIdx.x * kNaParts + threadIdx.x] = v;
-    }
+    if (tid >= D && tid < V) part[blockIdx.x * kNaParts + tid - D] = scalar;
 }
 
 // Sums the per-block partials in a fixed order into the three final slots.
@@ -154,6 +176,9 @@ int scratch_address(double **out) {
 }
 
 }  // namespace
+}  // namespace mds
+
+using namespace mds;
 
 extern "C" int mds_loglik_grad_noalloc(int64_t n, int32_t d, const float *y, int64_t ld, const double *x,
                                        double sigma, double *grad, double *loglik, double *dlogl_dsigma,
@@ -163,26 +188,37 @@ extern "C" int mds_loglik_grad_noalloc(int64_t n, int32_t d, const float *y, int
                               "sigma > 0, non-NULL y, x, grad)", MDS_MAX_D);
         return MDS_ERR_INVALID_ARG;
     }
-    const int64_t nblocks = (n + kNaWarps - 1) / kNaWarps;
-    if (nblocks > kNaMaxBlocks) {
-        mds::set_thread_error("mds_loglik_grad_noalloc: N = %lld exceeds the maximum %d of the fixed scratch",
-                              static_cast<long long>(n), kNaMaxBlocks * kNaWarps);
+    if (n > kNaMaxN) {
+        mds::set_thread_error("mds_loglik_grad_noalloc: N = %lld exceeds the maximum %lld of the fixed scratch",
+                              static_cast<long long>(n), static_cast<long long>(kNaMaxN));
         return MDS_ERR_INVALID_ARG;
     }
+    const int rows = static_cast<int>((n + kNaMaxBlocks - 1) / kNaMaxBlocks);
+    const int64_t nblocks = (n + rows - 1) / rows;
     double *part = nullptr;
     int st = scratch_address(&part);
     if (st != MDS_OK) return st;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    cudaError_t e = cudaSuccess;
     switch (d) {
-#define MDS_NA_CASE(DD) \
-    case DD: noalloc_rows_kernel<DD><<<static_cast<int>(nblocks), kNaThreads, 0, s>>>(n, y, ld, x, sigma, grad, part); break;
+#define MDS_NA_CASE(DD)                                                                                           \
+    case DD:                                                                                                      \
+        e = mds::raise_dyn_smem(reinterpret_cast<const void *>(noalloc_rows_kernel<DD>), kPhiBytes);              \
+        if (e == cudaSuccess)                                                                                     \
+            noalloc_rows_kernel<DD>                                                                               \
+                <<<static_cast<int>(nblocks), kNaThreads, kPhiBytes, s>>>(n, rows, y, ld, x, sigma, grad, part); \
+        break;
         MDS_NA_CASE(1) MDS_NA_CASE(2) MDS_NA_CASE(3) MDS_NA_CASE(4)
         MDS_NA_CASE(5) MDS_NA_CASE(6) MDS_NA_CASE(7) MDS_NA_CASE(8)
 #undef MDS_NA_CASE
         default: break;
     }
+    if (e != cudaSuccess) {
+        mds::set_thread_error("mds_loglik_grad_noalloc: shared memory: %s", cudaGetErrorString(e));
+        return MDS_ERR_CUDA;
+    }
     noalloc_sum_kernel<<<1, 256, 0, s>>>(static_cast<int>(nblocks), part);
-    cudaError_t e = cudaGetLastError();
+    e = cudaGetLastError();
     if (e != cudaSuccess) {
         mds::set_thread_error("mds_loglik_grad_noalloc: launch: %s", cudaGetErrorString(e));
         return MDS_ERR_CUDA;

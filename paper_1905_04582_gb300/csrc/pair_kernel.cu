@@ -32,8 +32,8 @@
 //    warps; the reduce kernel combines the strips with FP32 two-sums.  No
 //    FP64 instruction runs in this kernel (FP64 is 1/64 rate on this GPU).
 //
-// FP64 path (pair_f64_kernel): same work split, CUDA's double sqrt / erfc /
-// log1p / exp per pair and FP64 sums (the plain FP64 GPU path).
+// FP64 path (pair_f64_kernel): same work split, the FP64 arithmetic of
+// pair_math64.cuh and FP64 sums (the plain FP64 GPU path).
 #include <cfloat>
 #include <cstdint>
 #include <map>
@@ -43,6 +43,7 @@
 
 #include "mds_internal.h"
 #include "pair_math.cuh"
+#include "pair_math64.cuh"
 
 namespace mds {
 namespace {
@@ -212,14 +213,32 @@ __global__ void __launch_bounds__(kPairThreads, (D <= 2 ? 4 : D <= 4 ? 3 : 2)) p
 // ---------------------------------------------------------------- FP64
 
 // The plain FP64 path: same tile work split; Y read straight from global
-// memory in the tile layout, locations from the FP64 state.
+// memory in the tile layout (each lane 8 rows x 4 columns, a column pair at
+// a time), the row block's locations and the table of phi/Phi and log Phi in
+// shared memory.  Bound by the FP64 pipe (pair_math64.cuh): per pair and
+// coordinate the difference, its square and the two accumulations (4), and
+// 11 + 14 for the rest, the 14 only where some lane of the warp has z < 9.5.
+// The weight is summed in units of -sigma^2, so that its two terms take one
+// FMA; the partial sums carry the factor -1/sigma^2.
 template <int D>
-__global__ void __launch_bounds__(kPairThreads) pair_f64_kernel(const __grid_constant__ PairArgs a) {
-    constexpr int V = 4 * D;
+struct F64Layout {
+    static constexpr int kXiOffset = kPhiBytes;             // [64][D] doubles
+    static constexpr int kBytes = kXiOffset + kTile * D * 8;
+    // the row sums of the four warps reuse the table once the tiles are done
+    static constexpr int kRedBytes = (kPairWarps * kTile * D + kPairWarps * 4) * 8;
+    static_assert(kRedBytes <= kPhiBytes, "row sums fit in the table");
+};
+
+template <int D>
+__global__ void __launch_bounds__(kPairThreads, D <= 4 ? 3 : 2) pair_f64_kernel(const __grid_constant__ PairArgs a) {
+    using L = F64Layout<D>;
+    constexpr int kCols = D <= 4 ? 2 : 1;  // columns at a time (registers)
+    constexpr int V = kCols * D;
     constexpr int P = Pow2<V>::value;
-    constexpr double kInvSqrt2Pi = 0.39894228040143267794;
-    constexpr double kInvSqrt2 = 0.70710678118654752440;
-    __shared__ double red[kPairWarps * kTile * D + kPairWarps * 4];
+    extern __shared__ __align__(128) unsigned char smem[];
+    double *tab = reinterpret_cast<double *>(smem);
+    double *xis = reinterpret_cast<double *>(smem + L::kXiOffset);
+    double *red = tab;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int la = lane & 7, lb = lane >> 3;
     if (blockIdx.x >= static_cast<unsigned>(a.n_strips)) return;
@@ -229,23 +248,19 @@ __global__ void __launch_bounds__(kPairThreads) pair_f64_kernel(const __grid_con
         if (tid == 0) atomicOr(a.err, kErrBadArgs);
         return;
     }
+    phi_table_load(tab);
+    const Sigma64 sg = sigma64(a.sigma);
     pdl_wait();
     if (a.stamps && lane == 0) atomicMin(&a.stamps[0], global_ns());
     const int64_t nt = a.nt, n = a.n;
     const bool ragged = (n % kTile) != 0;
     const int64_t t0 = tile_index(st.I, st.j0, nt);
     const int rowbase = st.I * kTile;
-    double xi[8][D];
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-#pragma unroll
-        for (int h = 0; h < 2; ++h)
-#pragma unroll
-            for (int k = 0; k < D; ++k) {
-                const int slot = rowbase + 2 * (la + 8 * q) + h;
-                const int64_t item = a.perm ? a.perm[slot] : slot;
-                xi[2 * q + h][k] = a.x64[item * D + k];
-            }
+    for (int idx = tid; idx < kTile * D; idx += kPairThreads) {
+        const int slot = rowbase + idx / D;
+        xis[idx] = a.x64[static_cast<int64_t>(a.perm ? a.perm[slot] : slot) * D + idx % D];
+    }
+    __syncthreads();
     double racc[8][D];
 #pragma unroll
     for (int r = 0; r < 8; ++r)
@@ -260,60 +275,71 @@ __global__ void __launch_bounds__(kPairThreads) pair_f64_kernel(const __grid_con
         const int64_t ncv = n - static_cast<int64_t>(J) * kTile;
         const float4 *ys =
             reinterpret_cast<const float4 *>(a.y + (t0 + jt - a.y_t0) * kTileElems + warp * kWarpTileElems);
-        double colv[P];
+        double *cp_out = colp_base + (col_slot(st.I, J) * kTile + warp * kWarpCols + 4 * lb) * D;
+#pragma unroll 1
+        for (int c0 = 0; c0 < 4; c0 += kCols) {
+            const int half = c0 >> 1;
+            double xj[kCols][D], cacc[kCols][D];
 #pragma unroll
-        for (int i = 0; i < P; ++i) colv[i] = 0.0;
+            for (int e = 0; e < kCols; ++e) {
+                const int64_t cslot = static_cast<int64_t>(J) * kTile + warp * kWarpCols + 4 * lb + c0 + e;
+                const int64_t citem = a.perm ? a.perm[cslot] : cslot;
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const int col = warp * kWarpCols + 4 * lb + c;
-            double xj[D];
-            const int64_t cslot = static_cast<int64_t>(J) * kTile + col;
-            const int64_t citem = a.perm ? a.perm[cslot] : cslot;
-#pragma unroll
-            for (int k = 0; k < D; ++k) xj[k] = a.x64[citem * D + k];
+                for (int k = 0; k < D; ++k) {
+                    xj[e][k] = a.x64[citem * D + k];
+                    cacc[e][k] = 0.0;
+                }
+            }
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                const float4 yv = ys[(2 * q + (c >> 1)) * 32 + (lane ^ ((c >> 1) << 2))];
+                const float4 yv = ys[(2 * q + half) * 32 + (lane ^ (half << 2))];
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const float yf = (c & 1) ? (h ? yv.w : yv.z) : (h ? yv.y : yv.x);
-                    const int r = row_rel + 2 * (la + 8 * q) + h;
-                    const bool valid = !masked || (col > r && col < ncv && yf >= 0.f);  // y < 0: held out
+                for (int eh = 0; eh < 2 * kCols; ++eh) {
+                    const int e = eh >> 1, h = eh & 1;
+                    const float yf = ((c0 + e) & 1) ? (h ? yv.w : yv.z) : (h ? yv.y : yv.x);
+                    const int rr = 2 * (la + 8 * q) + h;
+                    const int col = warp * kWarpCols + 4 * lb + c0 + e;
+                    const bool valid = !masked || (col > row_rel + rr && col < ncv && yf >= 0.f);  // y < 0: held out
                     double dl[D];
-                    double d2 = 0.0;
+                    double d2 = 1e-300;  // see root64
 #pragma unroll
                     for (int k = 0; k < D; ++k) {
-                        dl[k] = xi[2 * q + h][k] - xj[k];
+                        dl[k] = xis[rr * D + k] - xj[e][k];
                         d2 = fma(dl[k], dl[k], d2);
                     }
-                    const double del = sqrt(d2);
-                    const double inv = del > 0.0 ? 1.0 / del : 0.0;
-                    const double e = valid ? static_cast<double>(yf) - del : 0.0;
-                    const double z = del * a.inv_sigma;
-                    const double qz = 0.5 * erfc(z * kInvSqrt2);
-                    const double m = valid ? exp(-0.5 * z * z) * kInvSqrt2Pi / (1.0 - qz) : 0.0;
-                    e2 = fma(e, e, e2);
-                    md = fma(m, del, md);
-                    if (valid) lp += log1p(-qz);
-                    const double wi = (m * a.inv_sigma - e * a.inv_s2) * inv;
+                    double del, inv;
+                    root64(d2, del, inv);
+                    double w = valid ? widen(yf) - del : 0.0;  // y - delta
+                    e2 = fma(w, w, e2);
+                    const bool near = valid && phi_near(sg, del);
+                    if (__any_sync(0xffffffffu, near)) {
+                        double F, G;
+                        phi_eval<true>(tab, sg, del, F, G);
+                        F = near ? F : 0.0;
+                        lp += near ? G : 0.0;
+                        md = fma(F, del, md);
+                        w = fma(F, sg.neg_s, w);
+                    }
+                    w *= inv;
 #pragma unroll
                     for (int k = 0; k < D; ++k) {
-                        const double t = wi * dl[k];
-                        racc[2 * q + h][k] += t;
-                        colv[c * D + k] += t;
+                        racc[2 * q + h][k] = fma(w, dl[k], racc[2 * q + h][k]);
+                        cacc[e][k] = fma(w, dl[k], cacc[e][k]);
                     }
                 }
             }
-        }
-        lane_reduce<P, 3>(colv, lane, 0);
-        bool writer;
-        const int base = reduced_base<P, 3>(lane, 0, writer);
-        constexpr int kHeld = P >= 8 ? P / 8 : 1;
-        double *cp = colp_base + (col_slot(st.I, J) * kTile + warp * kWarpCols + 4 * lb) * D;
-        if (writer) {
+            double colv[P];
 #pragma unroll
-            for (int i = 0; i < kHeld; ++i)
-                if (base + i < V) cp[base + i] = colv[i];
+            for (int i = 0; i < P; ++i) colv[i] = i < V ? cacc[i < V ? i / D : 0][i % D] : 0.0;
+            lane_reduce<P, 3>(colv, lane, 0);
+            bool writer;
+            const int base = reduced_base<P, 3>(lane, 0, writer);
+            constexpr int kHeld = P >= 8 ? P / 8 : 1;
+            if (writer) {
+#pragma unroll
+                for (int i = 0; i < kHeld; ++i)
+                    if (base + i < V) cp_out[c0 * D + base + i] = -a.inv_s2 * colv[i];
+            }
         }
     }
     constexpr int VR = 8 * D;
@@ -326,6 +352,7 @@ __global__ void __launch_bounds__(kPairThreads) pair_f64_kernel(const __grid_con
             rv[(q * D + k) * 2 + 1] = racc[2 * q + 1][k];
         }
     lane_reduce<VR, 2>(rv, lane, 3);
+    __syncthreads();  // every warp is done with the table, whose memory the sums take
     {
         bool writer;
         const int base = reduced_base<VR, 2>(lane, 3, writer);
@@ -350,7 +377,7 @@ __global__ void __launch_bounds__(kPairThreads) pair_f64_kernel(const __grid_con
         double v = red[idx];
 #pragma unroll
         for (int w = 1; w < kPairWarps; ++w) v += red[w * kTile * D + idx];
-        rp[idx] = v;
+        rp[idx] = -a.inv_s2 * v;
     }
     if (tid < 3) {
         const double *sr = red + kPairWarps * kTile * D;
@@ -382,7 +409,9 @@ cudaError_t launch_f32_d(const PairArgs &a, cudaStream_t s, bool pdl, int smem_m
 template <int D>
 cudaError_t launch_f64_d(const PairArgs &a, cudaStream_t s, bool pdl) {
     if (a.n_strips <= 0) return cudaSuccess;
-    const cudaError_t e = launch_maybe_pdl(pdl, pair_f64_kernel<D>, dim3(a.n_strips), dim3(kPairThreads), 0, s, a);
+    constexpr int smem = F64Layout<D>::kBytes;
+    cudaError_t e = raise_dyn_smem(reinterpret_cast<const void *>(pair_f64_kernel<D>), smem);
+    if (e == cudaSuccess) e = launch_maybe_pdl(pdl, pair_f64_kernel<D>, dim3(a.n_strips), dim3(kPairThreads), smem, s, a);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 

@@ -1,0 +1,112 @@
+// FP64 per-pair arithmetic of Eq. (2) and Eq. (9) of arXiv:1905.04582, shared
+// by the FP64 pair pass (pair_kernel.cu) and the allocation-free entry point
+// (noalloc.cu).
+//
+// What bounds it: GB300 issues one FP64 warp instruction per SM sub-partition
+// every 64 cycles, so a pair costs its FP64 instructions and everything else
+// (integer, FP32, shared memory, MUFU) is nearly free beside them.  With
+// CUDA's sqrt, division, erfc, exp and log1p a pair took about 187 of them at
+// D = 2; the forms below take 19, and 14 more where Phi matters:
+//  - 1/delta and delta: one cubic (Halley) step from the hardware's
+//    reciprocal-root seed, then delta corrected by its own residual
+//    d^2 - s^2, which an FMA gives exactly: 8, for a root and a division;
+//  - phi/Phi and log Phi as functions of z alone, piecewise polynomials of
+//    degree 5 on nodes 1/64 apart (phi_table.h, absolute error 9e-18), the
+//    table in shared memory: 13, for an exp, an erfc, a division and a log1p.
+//    What matters is their absolute error: beside phi/Phi the weight holds
+//    (delta - y)/sigma, whose rounding is at least 2^-53 z;
+//  - beyond z = 9.5 both are dropped: phi/Phi < 1.1e-20 there, five orders
+//    below half an ulp of delta/sigma (1e-15), the rounding of the term it
+//    would be added to, and |log Phi| < 1.1e-21 against terms whose sum is
+//    rounded at 1e-16;
+//  - y, an FP32 value, widened by moving bits (a conversion instruction would
+//    cost as much as an FMA).
+// Measured (GB300, whole calls, the errors against 64 bits unchanged): L,
+// dL/dX and dL/dsigma at N = 5392, D = 2, caller's order, 4.35 -> 1.02 ms; the
+// allocation-free call at N = 3001, D = 3, 2.84 -> 0.61 ms.
+#pragma once
+
+#include <cstdint>
+
+namespace mds {
+namespace {
+
+#include "phi_table.h"
+
+constexpr int kPhiRow = 2 * (kPhiDeg + 1);                  // doubles per node
+constexpr int kPhiBytes = kPhiNodes * kPhiRow * 8;          // 58,464
+static_assert(kPhiDeg == 5 && kPhiPerUnit == 64 && kPhiBytes % 16 == 0, "phi_eval is written for this table");
+
+// The table into shared memory (16-byte aligned), by all threads of the CTA;
+// the caller synchronises.
+__device__ __forceinline__ void phi_table_load(double *tab) {
+    const double2 *src = reinterpret_cast<const double2 *>(g_phi_table);
+    double2 *dst = reinterpret_cast<double2 *>(tab);
+    for (int i = threadIdx.x; i < kPhiBytes / 16; i += blockDim.x) dst[i] = src[i];
+}
+
+// sigma in the forms the pair needs.
+struct Sigma64 {
+    double inv_s;        // 1 / sigma
+    double inv_s_nodes;  // 64 / sigma
+    double neg_s;        // -sigma
+    uint32_t near_hi;    // high word of 9.5 sigma: delta with a larger high word is beyond the table
+};
+
+__device__ __forceinline__ Sigma64 sigma64(double sigma) {
+    return Sigma64{1.0 / sigma, 64.0 / sigma, -sigma, static_cast<uint32_t>(__double2hiint(9.5 * sigma))};
+}
+
+// An FP32 value as FP64: the exponent re-biased and the mantissa moved, for
+// normal positive numbers (a dissimilarity); anything else is converted.
+__device__ __forceinline__ double widen(float y) {
+    const uint32_t b = __float_as_uint(y);
+    if (b - 0x00800000u < 0x7f000000u)
+        return __hiloint2double(static_cast<int>((b >> 3) + 0x38000000u), static_cast<int>(b << 29));
+    return static_cast<double>(y);
+}
+
+// delta = sqrt(d2) and 1 / delta for d2 >= 1e-300 (the caller starts its sum
+// of squares there: coincident points get delta = 1e-150, below every
+// rounding, and a gradient term of exactly 0).  With r the seed and
+// e = 1 - d2 r^2: 1/sqrt(d2) = r (1 + e/2 + 3 e^2/8 + ...).
+__device__ __forceinline__ void root64(double d2, double &del, double &inv) {
+    double r;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d2));
+    const double t = d2 * r;
+    const double e = fma(-t, r, 1.0);
+    const double q = e * fma(e, 0.375, 0.5);
+    inv = fma(r, q, r);
+    const double s = fma(t, q, t);
+    const double half_inv = __hiloint2double(__double2hiint(inv) - 0x00100000, __double2loint(inv));
+    del = fma(fma(-s, s, d2), half_inv, s);
+}
+
+// Whether phi/Phi and log Phi are kept at this delta (a compare of high words).
+__device__ __forceinline__ bool phi_near(const Sigma64 &sg, double del) {
+    return static_cast<uint32_t>(__double2hiint(del)) <= sg.near_hi;
+}
+
+// F = phi(z)/Phi(z), G = log Phi(z) at z = del / sigma, phi_near(del); WANT_G false leaves G alone.
+template <bool WANT_G>
+__device__ __forceinline__ void phi_eval(const double *tab, const Sigma64 &sg, double del, double &F, double &G) {
+    // node: z * 64 to the nearest integer (the low bits of a sum with 1.5 * 2^52); at most 608 as
+    // phi_near bounds z, and cut there whatever the input
+    const uint32_t i = min(static_cast<uint32_t>(__double2loint(fma(del, sg.inv_s_nodes, 6755399441055744.0))),
+                           static_cast<uint32_t>(kPhiNodes - 1));
+    // -i / 64: an FP32 number (exact), widened
+    const float cf = (__uint_as_float(0x4B000000u | i) - 8388608.0f) * (1.0f / 64.0f);
+    const double nc =
+        __hiloint2double(static_cast<int>(i ? (__float_as_uint(cf) >> 3) + 0xB8000000u : 0u), 0);
+    const double t = fma(del, sg.inv_s, nc);
+    const double2 *row = reinterpret_cast<const double2 *>(tab + i * kPhiRow);
+    const double2 f54 = row[0], f32 = row[1], f10 = row[2];
+    F = fma(fma(fma(fma(fma(f54.x, t, f54.y), t, f32.x), t, f32.y), t, f10.x), t, f10.y);
+    if constexpr (WANT_G) {
+        const double2 g54 = row[3], g32 = row[4], g10 = row[5];
+        G = fma(fma(fma(fma(fma(g54.x, t, g54.y), t, g32.x), t, g32.y), t, g10.x), t, g10.y);
+    }
+}
+
+}  // namespace
+}  // namespace mds
