@@ -1633,8 +1633,9 @@ int create_ctx(int64_t n, int32_t d, uint32_t flags, bool alloc_y, mds_ctx **out
     if ((st = dev_alloc_t(c, &c->bad, sizeof(unsigned long long)))) return cleanup(st);
     if ((st = dev_alloc_t(c, &c->stamps, 2 * sizeof(unsigned long long)))) return cleanup(st);
     if ((st = dev_alloc_t(c, &c->pass_ns, 2 * sizeof(double)))) return cleanup(st);
-    const int64_t start_grid_max = (nd_pad + 4 * 256 - 1) / (4 * 256) + 1;
-    if ((st = dev_alloc_t(c, &c->e_start, start_grid_max * 2 * sizeof(double)))) return cleanup(st);
+    // two energy partials of every CTA of the trajectory-start kernel
+    if ((st = dev_alloc_t(c, &c->e_start, static_cast<size_t>(traj_start_grid(n, d)) * 2 * sizeof(double))))
+        return cleanup(st);
     if ((st = dev_alloc_t(c, &c->e_end, (c->nt * kReduceQuarters + 1) * 2 * sizeof(double)))) return cleanup(st);
     if ((st = dev_alloc(c, &c->stage, nd_pad * sizeof(double)))) return cleanup(st);
     if (cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking) != cudaSuccess ||
