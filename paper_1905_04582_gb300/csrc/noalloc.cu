@@ -91,14 +91,13 @@ __device__ __forceinline__ void row_part(const double *tab, const Sigma64 &sg, c
 
 template <int D>
 __global__ void __launch_bounds__(kNaThreads, 3) noalloc_rows_kernel(int64_t n, int rows, const float *y, int64_t ld,
-                                                                     const double *x, double sigma, double *grad,
+                                                                     const double *x, Sigma64 sg, double *grad,
                                                                      double *part) {
     constexpr int V = D + 3, P = Pow2<V>::value;
     extern __shared__ __align__(16) unsigned char na_smem[];
     double *tab = reinterpret_cast<double *>(na_smem);
     __shared__ double red[kNaWarps][V];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const Sigma64 sg = sigma64(sigma);
     phi_table_load(tab);
     __syncthreads();
     double scalar = 0.0;  // threads D .. D + 2: the block's sums of the scalar terms
@@ -200,13 +199,14 @@ extern "C" int mds_loglik_grad_noalloc(int64_t n, int32_t d, const float *y, int
     if (st != MDS_OK) return st;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     cudaError_t e = cudaSuccess;
+    const Sigma64 sg = sigma64(sigma);
     switch (d) {
 #define MDS_NA_CASE(DD)                                                                                           \
     case DD:                                                                                                      \
         e = mds::raise_dyn_smem(reinterpret_cast<const void *>(noalloc_rows_kernel<DD>), kPhiBytes);              \
         if (e == cudaSuccess)                                                                                     \
             noalloc_rows_kernel<DD>                                                                               \
-                <<<static_cast<int>(nblocks), kNaThreads, kPhiBytes, s>>>(n, rows, y, ld, x, sigma, grad, part); \
+                <<<static_cast<int>(nblocks), kNaThreads, kPhiBytes, s>>>(n, rows, y, ld, x, sg, grad, part);    \
         break;
         MDS_NA_CASE(1) MDS_NA_CASE(2) MDS_NA_CASE(3) MDS_NA_CASE(4)
         MDS_NA_CASE(5) MDS_NA_CASE(6) MDS_NA_CASE(7) MDS_NA_CASE(8)

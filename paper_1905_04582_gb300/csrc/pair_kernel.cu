@@ -230,7 +230,7 @@ struct F64Layout {
 };
 
 template <int D>
-__global__ void __launch_bounds__(kPairThreads, D <= 4 ? 3 : 2) pair_f64_kernel(const __grid_constant__ PairArgs a) {
+__global__ void __launch_bounds__(kPairThreads, D <= 4 ? 3 : 2) pair_f64_kernel(const __grid_constant__ PairArgs a, const __grid_constant__ Sigma64 sg) {
     using L = F64Layout<D>;
     constexpr int kCols = D <= 4 ? 2 : 1;  // columns at a time (registers)
     constexpr int V = kCols * D;
@@ -249,7 +249,6 @@ __global__ void __launch_bounds__(kPairThreads, D <= 4 ? 3 : 2) pair_f64_kernel(
         return;
     }
     phi_table_load(tab);
-    const Sigma64 sg = sigma64(a.sigma);
     pdl_wait();
     if (a.stamps && lane == 0) atomicMin(&a.stamps[0], global_ns());
     const int64_t nt = a.nt, n = a.n;
@@ -411,7 +410,7 @@ cudaError_t launch_f64_d(const PairArgs &a, cudaStream_t s, bool pdl) {
     if (a.n_strips <= 0) return cudaSuccess;
     constexpr int smem = F64Layout<D>::kBytes;
     cudaError_t e = raise_dyn_smem(reinterpret_cast<const void *>(pair_f64_kernel<D>), smem);
-    if (e == cudaSuccess) e = launch_maybe_pdl(pdl, pair_f64_kernel<D>, dim3(a.n_strips), dim3(kPairThreads), smem, s, a);
+    if (e == cudaSuccess) e = launch_maybe_pdl(pdl, pair_f64_kernel<D>, dim3(a.n_strips), dim3(kPairThreads), smem, s, a, sigma64(a.sigma));
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 

@@ -1,6 +1,6 @@
 // FP64 per-pair arithmetic of Eq. (2) and Eq. (9) of arXiv:1905.04582, shared
-// by the FP64 pair pass (pair_kernel.cu) and the allocation-free entry point
-// (noalloc.cu).
+// by the FP64 pair pass (pair_kernel.cu), the allocation-free entry point
+// (noalloc.cu) and the held-out densities (heldout.cu).
 //
 // What bounds it: GB300 issues one FP64 warp instruction per SM sub-partition
 // every 64 cycles, so a pair costs its FP64 instructions and everything else
@@ -27,6 +27,7 @@
 #pragma once
 
 #include <cstdint>
+#include <cstring>
 
 namespace mds {
 namespace {
@@ -53,8 +54,13 @@ struct Sigma64 {
     uint32_t near_hi;    // high word of 9.5 sigma: delta with a larger high word is beyond the table
 };
 
-__device__ __forceinline__ Sigma64 sigma64(double sigma) {
-    return Sigma64{1.0 / sigma, 64.0 / sigma, -sigma, static_cast<uint32_t>(__double2hiint(9.5 * sigma))};
+// On the host, for a kernel argument: three divisions a thread would cost as
+// much as a pair or two.
+inline Sigma64 sigma64(double sigma) {
+    const double near = 9.5 * sigma;
+    uint64_t bits;
+    std::memcpy(&bits, &near, sizeof(bits));
+    return Sigma64{1.0 / sigma, 64.0 / sigma, -sigma, static_cast<uint32_t>(bits >> 32)};
 }
 
 // An FP32 value as FP64: the exponent re-biased and the mantissa moved, for
@@ -64,6 +70,15 @@ __device__ __forceinline__ double widen(float y) {
     if (b - 0x00800000u < 0x7f000000u)
         return __hiloint2double(static_cast<int>((b >> 3) + 0x38000000u), static_cast<int>(b << 29));
     return static_cast<double>(y);
+}
+
+// The same for a number of either sign (a coordinate).
+__device__ __forceinline__ double widen_signed(float v) {
+    const uint32_t b = __float_as_uint(v), m = b & 0x7fffffffu;
+    if (m - 0x00800000u < 0x7f000000u)
+        return __hiloint2double(static_cast<int>((b & 0x80000000u) | ((m >> 3) + 0x38000000u)),
+                                static_cast<int>(b << 29));
+    return static_cast<double>(v);
 }
 
 // delta = sqrt(d2) and 1 / delta for d2 >= 1e-300 (the caller starts its sum
@@ -87,10 +102,9 @@ __device__ __forceinline__ bool phi_near(const Sigma64 &sg, double del) {
     return static_cast<uint32_t>(__double2hiint(del)) <= sg.near_hi;
 }
 
-// F = phi(z)/Phi(z), G = log Phi(z) at z = del / sigma, phi_near(del); WANT_G false leaves G alone.
-template <bool WANT_G>
-__device__ __forceinline__ void phi_eval(const double *tab, const Sigma64 &sg, double del, double &F, double &G) {
-    // node: z * 64 to the nearest integer (the low bits of a sum with 1.5 * 2^52); at most 608 as
+// The node of z = del / sigma, phi_near(del): its index, and t = z - i / 64.
+__device__ __forceinline__ uint32_t phi_node(const Sigma64 &sg, double del, double &t) {
+    // z * 64 to the nearest integer (the low bits of a sum with 1.5 * 2^52); at most 608 as
     // phi_near bounds z, and cut there whatever the input
     const uint32_t i = min(static_cast<uint32_t>(__double2loint(fma(del, sg.inv_s_nodes, 6755399441055744.0))),
                            static_cast<uint32_t>(kPhiNodes - 1));
@@ -98,14 +112,29 @@ __device__ __forceinline__ void phi_eval(const double *tab, const Sigma64 &sg, d
     const float cf = (__uint_as_float(0x4B000000u | i) - 8388608.0f) * (1.0f / 64.0f);
     const double nc =
         __hiloint2double(static_cast<int>(i ? (__float_as_uint(cf) >> 3) + 0xB8000000u : 0u), 0);
-    const double t = fma(del, sg.inv_s, nc);
-    const double2 *row = reinterpret_cast<const double2 *>(tab + i * kPhiRow);
-    const double2 f54 = row[0], f32 = row[1], f10 = row[2];
-    F = fma(fma(fma(fma(fma(f54.x, t, f54.y), t, f32.x), t, f32.y), t, f10.x), t, f10.y);
-    if constexpr (WANT_G) {
-        const double2 g54 = row[3], g32 = row[4], g10 = row[5];
-        G = fma(fma(fma(fma(fma(g54.x, t, g54.y), t, g32.x), t, g32.y), t, g10.x), t, g10.y);
-    }
+    t = fma(del, sg.inv_s, nc);
+    return i;
+}
+
+__device__ __forceinline__ double phi_poly(const double2 *c, double t) {
+    const double2 c54 = c[0], c32 = c[1], c10 = c[2];
+    return fma(fma(fma(fma(fma(c54.x, t, c54.y), t, c32.x), t, c32.y), t, c10.x), t, c10.y);
+}
+
+// F = phi(z)/Phi(z), G = log Phi(z) at z = del / sigma, phi_near(del); WANT_G false leaves G alone.
+template <bool WANT_G>
+__device__ __forceinline__ void phi_eval(const double *tab, const Sigma64 &sg, double del, double &F, double &G) {
+    double t;
+    const double2 *row = reinterpret_cast<const double2 *>(tab + phi_node(sg, del, t) * kPhiRow);
+    F = phi_poly(row, t);
+    if constexpr (WANT_G) G = phi_poly(row + 3, t);
+}
+
+// log Phi(z) alone.
+__device__ __forceinline__ double phi_log(const double *tab, const Sigma64 &sg, double del) {
+    double t;
+    const uint32_t i = phi_node(sg, del, t);
+    return phi_poly(reinterpret_cast<const double2 *>(tab + i * kPhiRow) + 3, t);
 }
 
 }  // namespace
