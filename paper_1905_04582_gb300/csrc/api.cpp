@@ -116,6 +116,8 @@ struct mds_ctx {
     double *scal = nullptr;
     int64_t *counters = nullptr;
     unsigned *err = nullptr;
+    bool shared_words = false;  // err, scal and counters belong to the batch
+    HostPub *pub = nullptr;   // pinned: error bits and scalars that the device hands back
     unsigned long long *bad = nullptr;
     double *e_start = nullptr, *e_end = nullptr;
     void *stage = nullptr;    // conversion staging (n_pad * D doubles)
@@ -282,10 +284,24 @@ int err_status(mds_ctx *c, unsigned h, const char *what) {
 }
 
 // Read and clear the device error word; map it to a status.
+int published_status(mds_ctx *c, const char *what);
 int check_device_err(mds_ctx *c, const char *what) {
-    unsigned h = 0;
-    CU(cudaMemcpyAsync(&h, c->err, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream));
+    CU(cudaMemcpyAsync(&c->pub->err, c->err, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream));
     CU(cudaStreamSynchronize(c->stream));
+    return published_status(c, what);
+}
+
+// The error word and the scalars (and the gradient, into dst) to the host.
+int publish(mds_ctx *c, void *dst = nullptr, bool dst_f64 = false) {
+    cudaError_t e = launch_publish(c->grad, !c->fp64, dst, dst_f64, c->n * c->d, c->err, c->scal, c->pub, c->stream);
+    if (e != cudaSuccess) return fail(c, MDS_ERR_CUDA, "publish launch: %s", cudaGetErrorString(e));
+    return MDS_OK;
+}
+
+// The error word as it was handed back (c->pub->err, after the wait): cleared
+// on the device, and mapped to a status.
+int published_status(mds_ctx *c, const char *what) {
+    const unsigned h = c->pub->err;
     if (h == 0) return MDS_OK;
     CU(cudaMemsetAsync(c->err, 0, sizeof(unsigned), c->stream));
     CU(cudaStreamSynchronize(c->stream));
@@ -1090,8 +1106,9 @@ int autotune(mds_ctx *c) {
     return MDS_OK;
 }
 
-// Evaluate at the current x (gradient + scalars) and wait.
-int evaluate(mds_ctx *c) {
+// Evaluate at the current x (gradient + scalars) and wait; the scalars are
+// then in c->pub, and the gradient in dst (device memory, if given).
+int evaluate(mds_ctx *c, void *dst = nullptr, bool dst_f64 = false) {
     CHECK(ready(c));
     CHECK(autotune(c));
     if (fault_is("timeout")) {
@@ -1099,8 +1116,9 @@ int evaluate(mds_ctx *c) {
         if (e != cudaSuccess) return fail(c, MDS_ERR_CUDA, "wait probe: %s", cudaGetErrorString(e));
     }
     CHECK(enqueue_pass(c, kModeEval, 0.0, c->stream, fault_is("nan")));
-    CU(cudaGetLastError());
-    CHECK(check_device_err(c, "evaluation"));
+    CHECK(publish(c, dst, dst_f64));
+    CU(cudaStreamSynchronize(c->stream));
+    CHECK(published_status(c, "evaluation"));
     if (c->profiling) CHECK(harvest_prof(c));
     c->grad_valid = true;
     return MDS_OK;
@@ -1162,6 +1180,19 @@ int stage_in(mds_ctx *c, const void *src, int dtype, int where, int64_t count, c
     }
     CU(cudaMemcpyAsync(c->stage, src, count * eb, cudaMemcpyHostToDevice, c->stream));
     *dev = c->stage;
+    return MDS_OK;
+}
+
+int valid_enums(mds_ctx *c, int dtype, int where);
+
+// The caller's momenta into the state, without a wait (the caller waits
+// before its own return, so that the source is no longer read then).
+int queue_momentum(mds_ctx *c, const void *p, int dtype, int where) {
+    CHECK(valid_enums(c, dtype, where));
+    const void *dev = nullptr;
+    CHECK(stage_in(c, p, dtype, where, c->n * c->d, &dev));
+    cudaError_t e = launch_convert(dev, dtype == MDS_F64, c->p, c->fp64, c->n * c->d, c->stream);
+    if (e != cudaSuccess) return fail(c, MDS_ERR_CUDA, "set_momentum: %s", cudaGetErrorString(e));
     return MDS_OK;
 }
 
@@ -1630,6 +1661,13 @@ int create_ctx(int64_t n, int32_t d, uint32_t flags, bool alloc_y, mds_ctx **out
     if ((st = dev_alloc_t(c, &c->scal, kScalars * sizeof(double)))) return cleanup(st);
     if ((st = dev_alloc_t(c, &c->counters, kCounters * sizeof(int64_t)))) return cleanup(st);
     if ((st = dev_alloc_t(c, &c->err, sizeof(unsigned)))) return cleanup(st);
+    if (cudaMallocHost(&c->pub, sizeof(HostPub)) != cudaSuccess) {
+        cudaGetLastError();
+        c->pub = nullptr;
+        c->last_error = "pinned host allocation failed";
+        return cleanup(MDS_ERR_OOM);
+    }
+    *c->pub = HostPub{};
     if ((st = dev_alloc_t(c, &c->bad, sizeof(unsigned long long)))) return cleanup(st);
     if ((st = dev_alloc_t(c, &c->stamps, 2 * sizeof(unsigned long long)))) return cleanup(st);
     if ((st = dev_alloc_t(c, &c->pass_ns, 2 * sizeof(double)))) return cleanup(st);
@@ -1680,6 +1718,11 @@ int mds_destroy(mds_ctx *c) {
     if (c->stream) cudaStreamSynchronize(c->stream);
     if (c->graph) cudaGraphExecDestroy(c->graph);
     if (!c->y_owned) c->y = nullptr;
+    if (c->shared_words) {
+        c->err = nullptr;
+        c->scal = nullptr;
+        c->counters = nullptr;
+    }
     void *bufs[] = {c->y,        c->x,        c->p,         c->x0,       c->xrow,      c->xcol,
                     c->split,    c->xmax_bits, c->grad,     c->grad0,    c->col_part,  c->row_part,
                     c->scal_part, c->strips,  c->row_first, c->scal,     c->counters,  c->err,
@@ -1691,6 +1734,7 @@ int mds_destroy(mds_ctx *c) {
     for (void *b : ho_bufs) dev_free(b);
     for (void *b : c->tree_bufs) dev_free(b);
     if (c->host_stage) cudaFreeHost(c->host_stage);
+    if (c->pub) cudaFreeHost(c->pub);
     if (c->shard_hsend) cudaFreeHost(c->shard_hsend);
     if (c->shard_hrecv) cudaFreeHost(c->shard_hrecv);
     if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
@@ -1823,31 +1867,17 @@ int mds_set_locations(mds_ctx *c, const void *x, int dtype, int where) {
     CHECK(valid_enums(c, dtype, where));
     const void *dev = nullptr;
     CHECK(stage_in(c, x, dtype, where, c->n * c->d, &dev));
-    CU(cudaMemsetAsync(c->err, 0, sizeof(unsigned), c->stream));
-    if (!c->fp64) {
-        // max |x| of the incoming values; the set_x kernel derives the
-        // quantum of the exact-difference split from it on the device
-        CU(cudaMemsetAsync(c->xmax_bits, 0, sizeof(unsigned), c->stream));
-        cudaError_t e = launch_xmax(dev, dtype == MDS_F64, c->n * c->d, c->xmax_bits, c->stream);
-        if (e != cudaSuccess) return fail(c, MDS_ERR_CUDA, "set_locations: %s", cudaGetErrorString(e));
-    }
-    cudaError_t e = launch_set_x(dev, dtype == MDS_F64, c->n, c->n_pad, c->d, c->fp64, xstate(c), c->err, c->stream);
+    c->pub->err = 0;
+    cudaError_t e =
+        launch_set_x(dev, dtype == MDS_F64, c->n, c->n_pad, c->d, c->fp64, xstate(c), c->err, c->pub, c->stream);
     if (e != cudaSuccess) return fail(c, MDS_ERR_CUDA, "set_locations: %s", cudaGetErrorString(e));
-    // the one wait of the call: the error word (non-finite entry, range)
-    unsigned h = 0;
-    CU(cudaMemcpyAsync(&h, c->err, sizeof(h), cudaMemcpyDeviceToHost, c->stream));
+    // the one wait of the call: its error bits (non-finite entry, range)
     CU(cudaStreamSynchronize(c->stream));
+    const unsigned h = c->pub->err;
     if (h) {
-        unsigned bits = 0;
-        if (!c->fp64) CU(cudaMemcpyAsync(&bits, c->xmax_bits, sizeof(bits), cudaMemcpyDeviceToHost, c->stream));
-        CU(cudaMemsetAsync(c->err, 0, sizeof(unsigned), c->stream));
-        CU(cudaStreamSynchronize(c->stream));
-        if (h & kErrRange) {
-            // nothing was written: the previous locations stay in place
-            float m;
-            std::memcpy(&m, &bits, sizeof(m));
-            return fail(c, MDS_ERR_INVALID_ARG, "locations out of the FP32C range (max |x| = %g)", m);
-        }
+        // out of range: nothing was written, the previous locations stay in place
+        if (h & kErrRange)
+            return fail(c, MDS_ERR_INVALID_ARG, "locations out of the FP32C range (max |x| = %g)", c->pub->xmax);
         c->have_x = false;
         return fail(c, MDS_ERR_INVALID_ARG, "X has a NaN or Inf entry");
     }
@@ -1891,10 +1921,13 @@ int mds_set_prior(mds_ctx *c, double lambda) {
 int mds_log_likelihood(mds_ctx *c, double *loglik, double *sum_r) {
     CHECK(check_ctx(c));
     if (!loglik && !sum_r) return fail(c, MDS_ERR_INVALID_ARG, "no output requested");
-    if (!c->grad_valid) CHECK(evaluate(c));
-    double s[kScalars];
-    CU(cudaMemcpyAsync(s, c->scal, sizeof(s), cudaMemcpyDeviceToHost, c->stream));
-    CU(cudaStreamSynchronize(c->stream));
+    if (!c->grad_valid) {
+        CHECK(evaluate(c));
+    } else {
+        CU(cudaMemcpyAsync(c->pub->scal, c->scal, kScalars * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+        CU(cudaStreamSynchronize(c->stream));
+    }
+    const double *s = c->pub->scal;
     if (loglik) *loglik = s[kLogLik];
     if (sum_r) *sum_r = s[kSumR];
     if (!std::isfinite(s[kLogLik])) return fail(c, MDS_ERR_NONFINITE, "log-likelihood is not finite");
@@ -1904,26 +1937,24 @@ int mds_log_likelihood(mds_ctx *c, double *loglik, double *sum_r) {
 int mds_gradient(mds_ctx *c, double *loglik, void *grad, int dtype, int where, double *dsigma) {
     CHECK(check_ctx(c));
     if (grad) CHECK(valid_enums(c, dtype, where));
-    CHECK(evaluate(c));
-    if (grad) CHECK(copy_out(c, c->grad, c->fp64 ? 1 : 2, grad, dtype, where, c->n * c->d));
-    if (loglik || dsigma) {
-        double s[kScalars];
-        CU(cudaMemcpyAsync(s, c->scal, sizeof(s), cudaMemcpyDeviceToHost, c->stream));
+    const bool dst_f64 = dtype == MDS_F64;
+    if (grad && where == MDS_HOST) {
+        // through the staging buffer; nothing reaches the caller before the evaluation is known to be good
+        CHECK(evaluate(c, c->stage, dst_f64));
+        CU(cudaMemcpyAsync(grad, c->stage, c->n * c->d * (dst_f64 ? 8 : 4), cudaMemcpyDeviceToHost, c->stream));
         CU(cudaStreamSynchronize(c->stream));
-        if (loglik) *loglik = s[kLogLik];
-        if (dsigma) *dsigma = s[kDSigma];
+    } else {
+        CHECK(evaluate(c, grad, dst_f64));
     }
+    if (loglik) *loglik = c->pub->scal[kLogLik];
+    if (dsigma) *dsigma = c->pub->scal[kDSigma];
     return MDS_OK;
 }
 
 int mds_set_momentum(mds_ctx *c, const void *p, int dtype, int where) {
     CHECK(check_ctx(c));
     if (!p) return fail(c, MDS_ERR_INVALID_ARG, "p is NULL");
-    CHECK(valid_enums(c, dtype, where));
-    const void *dev = nullptr;
-    CHECK(stage_in(c, p, dtype, where, c->n * c->d, &dev));
-    cudaError_t e = launch_convert(dev, dtype == MDS_F64, c->p, c->fp64, c->n * c->d, c->stream);
-    if (e != cudaSuccess) return fail(c, MDS_ERR_CUDA, "set_momentum: %s", cudaGetErrorString(e));
+    CHECK(queue_momentum(c, p, dtype, where));
     CU(cudaStreamSynchronize(c->stream));
     return MDS_OK;
 }
@@ -1940,18 +1971,15 @@ int mds_leapfrog(mds_ctx *c, int n_steps, double eps, const void *p0, int p0_dty
     if (n_steps < 0) return fail(c, MDS_ERR_INVALID_ARG, "n_steps must be >= 0");
     if (!std::isfinite(eps)) return fail(c, MDS_ERR_INVALID_ARG, "eps must be finite");
     CHECK(ready(c));
-    if (p0) CHECK(mds_set_momentum(c, p0, p0_dtype, p0_where));
+    if (p0) CHECK(queue_momentum(c, p0, p0_dtype, p0_where));
     if (!c->grad_valid) CHECK(evaluate(c));
     CHECK(autotune(c));
     CHECK(enqueue_trajectory(c, n_steps, eps, 0, 1, 0, 0, c->stream));
-    CHECK(check_device_err(c, "leapfrog"));
+    CHECK(publish(c));
+    CU(cudaStreamSynchronize(c->stream));
+    CHECK(published_status(c, "leapfrog"));
     if (c->profiling) CHECK(harvest_prof(c));
-    if (dh) {
-        double s[kScalars];
-        CU(cudaMemcpyAsync(s, c->scal, sizeof(s), cudaMemcpyDeviceToHost, c->stream));
-        CU(cudaStreamSynchronize(c->stream));
-        *dh = s[kLastDH];
-    }
+    if (dh) *dh = c->pub->scal[kLastDH];
     return MDS_OK;
 }
 
@@ -2168,10 +2196,7 @@ int mds_sigma_mh(mds_ctx *c, int n_iter, double step, double shape, double rate,
     };
     auto eval_ll = [&](double *ll) -> int {
         CHECK(evaluate(c));
-        double s[kScalars];
-        CU(cudaMemcpyAsync(s, c->scal, sizeof(s), cudaMemcpyDeviceToHost, c->stream));
-        CU(cudaStreamSynchronize(c->stream));
-        *ll = s[kLogLik];
+        *ll = c->pub->scal[kLogLik];
         return MDS_OK;
     };
     double ll = 0.0;
@@ -3057,6 +3082,15 @@ struct mds_batch {
     uint64_t gen = 1;
     cudaGraphExec_t graph = nullptr;
     std::tuple<uint64_t, int> graph_key{};
+    // the chains' scalars, counters and error words, each chain's after the
+    // other's, so that one copy or memset serves all of them
+    double *scal_all = nullptr;
+    int64_t *counters_all = nullptr;
+    unsigned *err_all = nullptr;
+    void *host = nullptr;      // pinned read-back buffer (grown on demand, kept)
+    size_t host_bytes = 0;
+    std::vector<double> eps;   // step of each dataset in the reduction's table
+    std::vector<unsigned char> sent[5];  // the device tables as uploaded
     std::string last_error = "no error";
 };
 
@@ -3115,6 +3149,41 @@ int bdev_alloc(mds_batch *b, P **p, size_t bytes) {
     return MDS_OK;
 }
 
+// A device table from its host copy, if it differs from what the device holds
+// (a copy from pageable memory has left the source when the call returns).
+template <typename T>
+int batch_upload(mds_batch *b, int slot, T *dev, const std::vector<T> &v) {
+    const size_t bytes = v.size() * sizeof(T);
+    std::vector<unsigned char> &sent = b->sent[slot];
+    if (sent.size() == bytes && (bytes == 0 || std::memcmp(sent.data(), v.data(), bytes) == 0)) return MDS_OK;
+    sent.clear();
+    if (bytes) BCU(cudaMemcpyAsync(dev, v.data(), bytes, cudaMemcpyHostToDevice, b->stream));
+    const unsigned char *src = reinterpret_cast<const unsigned char *>(v.data());
+    sent.assign(src, src + bytes);
+    return MDS_OK;
+}
+
+// Pinned host memory for read-backs.
+int batch_host(mds_batch *b, size_t bytes) {
+    if (bytes <= b->host_bytes) return MDS_OK;
+    if (b->host) {
+        BCU(cudaStreamSynchronize(b->stream));
+        cudaFreeHost(b->host);
+        b->host = nullptr;
+        b->host_bytes = 0;
+    }
+    const size_t nb = std::max<size_t>(bytes, 4096);
+    BCU(cudaMallocHost(&b->host, nb));
+    b->host_bytes = nb;
+    return MDS_OK;
+}
+
+double eps_of(const mds_batch *b, int g) {
+    int dd = 0;
+    while (dd + 1 < b->n_data && g >= b->chain0[dd + 1]) ++dd;
+    return b->eps[dd];
+}
+
 // Bring every chain to the batch strip length, refresh the location splits,
 // and (re)build the device tables of the batched pair pass and reduction.
 int batch_tables(mds_batch *b, int strip) {
@@ -3163,13 +3232,14 @@ int batch_tables(mds_batch *b, int strip) {
         const mds_ctx *c = b->ctx[g];
         ch[g] = BatchChain{c->xrow, c->xcol, static_cast<float *>(c->row_part), static_cast<float *>(c->col_part),
                            static_cast<float *>(c->scal_part)};
-        rc[g] = reduce_args(c, kModeEval, 0.0);
+        rc[g] = reduce_args(c, kModeEval, eps_of(b, g));
         for (int J = 0; J < c->nt * kReduceQuarters; ++J) jobs.push_back(make_int2(g, J));
         jobs.push_back(make_int2(g, -1));
     }
     if (st.size() > b->strips_cap) {
         if (b->strips_dev) cudaFree(b->strips_dev);
         b->strips_dev = nullptr;
+        b->sent[2].clear();
         CHECK(bdev_alloc(b, &b->strips_dev, st.size() * sizeof(BatchStrip)));
         b->strips_cap = st.size();
         b->gen++;
@@ -3177,16 +3247,16 @@ int batch_tables(mds_batch *b, int strip) {
     if (jobs.size() > b->jobs_cap) {
         if (b->jobs) cudaFree(b->jobs);
         b->jobs = nullptr;
+        b->sent[3].clear();
         CHECK(bdev_alloc(b, &b->jobs, jobs.size() * sizeof(int2)));
         b->jobs_cap = jobs.size();
         b->gen++;
     }
-    BCU(cudaMemcpyAsync(b->ds_dev, ds.data(), ds.size() * sizeof(BatchDataset), cudaMemcpyHostToDevice, b->stream));
-    BCU(cudaMemcpyAsync(b->ch_dev, ch.data(), ch.size() * sizeof(BatchChain), cudaMemcpyHostToDevice, b->stream));
-    BCU(cudaMemcpyAsync(b->strips_dev, st.data(), st.size() * sizeof(BatchStrip), cudaMemcpyHostToDevice, b->stream));
-    BCU(cudaMemcpyAsync(b->jobs, jobs.data(), jobs.size() * sizeof(int2), cudaMemcpyHostToDevice, b->stream));
-    BCU(cudaMemcpyAsync(b->rcfg, rc.data(), rc.size() * sizeof(ReduceArgs), cudaMemcpyHostToDevice, b->stream));
-    BCU(cudaStreamSynchronize(b->stream));
+    CHECK(batch_upload(b, 0, b->ds_dev, ds));
+    CHECK(batch_upload(b, 1, b->ch_dev, ch));
+    CHECK(batch_upload(b, 2, b->strips_dev, st));
+    CHECK(batch_upload(b, 3, b->jobs, jobs));
+    CHECK(batch_upload(b, 4, b->rcfg, rc));
     if (static_cast<int32_t>(st.size()) != b->n_strips || static_cast<int32_t>(jobs.size()) != b->n_jobs ||
         strip != b->strip)
         b->gen++;
@@ -3233,10 +3303,25 @@ int batch_enqueue_pass(mds_batch *b, int mode, cudaStream_t s) {
     return MDS_OK;
 }
 
-int batch_check_errors(mds_batch *b, const char *what) {
-    BCU(cudaStreamSynchronize(b->stream));
-    for (mds_ctx *c : b->ctx) CHECK(bpass(b, c, check_device_err(c, what)));
+// The chains' error words (host copies, after a wait): the first that is set
+// is cleared and mapped to the status.
+int batch_status(mds_batch *b, const unsigned *words, const char *what) {
+    for (size_t g = 0; g < b->ctx.size(); ++g) {
+        if (words[g] == 0) continue;
+        mds_ctx *c = b->ctx[g];
+        c->pub->err = words[g];
+        CHECK(bpass(b, c, published_status(c, what)));
+    }
     return MDS_OK;
+}
+
+int batch_check_errors(mds_batch *b, const char *what) {
+    const size_t total = b->ctx.size();
+    CHECK(batch_host(b, total * sizeof(unsigned)));
+    unsigned *words = static_cast<unsigned *>(b->host);
+    BCU(cudaMemcpyAsync(words, b->err_all, total * sizeof(unsigned), cudaMemcpyDeviceToHost, b->stream));
+    BCU(cudaStreamSynchronize(b->stream));
+    return batch_status(b, words, what);
 }
 
 std::mutex g_btune_mu;
@@ -3360,6 +3445,27 @@ int mds_batch_create(int32_t n_data, const int64_t *n, int32_t d, const int32_t 
     bool ev_ok = cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking) == cudaSuccess &&
                  cudaEventCreate(&b->ev0) == cudaSuccess && cudaEventCreate(&b->ev1) == cudaSuccess &&
                  cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming) == cudaSuccess;
+    if ((st = bdev_alloc(b, &b->scal_all, static_cast<size_t>(total) * kScalars * sizeof(double)))) return cleanup(st);
+    if ((st = bdev_alloc(b, &b->counters_all, static_cast<size_t>(total) * kCounters * sizeof(int64_t))))
+        return cleanup(st);
+    if ((st = bdev_alloc(b, &b->err_all, static_cast<size_t>(total) * sizeof(unsigned)))) return cleanup(st);
+    b->eps.assign(n_data, 0.0);
+    if (cudaMemset(b->scal_all, 0, static_cast<size_t>(total) * kScalars * sizeof(double)) != cudaSuccess ||
+        cudaMemset(b->counters_all, 0, static_cast<size_t>(total) * kCounters * sizeof(int64_t)) != cudaSuccess ||
+        cudaMemset(b->err_all, 0, static_cast<size_t>(total) * sizeof(unsigned)) != cudaSuccess) {
+        b->last_error = "initial memset failed";
+        return cleanup(MDS_ERR_CUDA);
+    }
+    for (int g = 0; g < total; ++g) {
+        mds_ctx *x = b->ctx[g];
+        dev_free(x->scal);
+        dev_free(x->counters);
+        dev_free(x->err);
+        x->scal = b->scal_all + static_cast<size_t>(g) * kScalars;
+        x->counters = b->counters_all + static_cast<size_t>(g) * kCounters;
+        x->err = b->err_all + g;
+        x->shared_words = true;
+    }
     b->joins.assign(b->ctx.size(), nullptr);
     for (size_t g = 0; ev_ok && g < b->ctx.size(); ++g)
         ev_ok = cudaEventCreateWithFlags(&b->joins[g], cudaEventDisableTiming) == cudaSuccess;
@@ -3381,6 +3487,10 @@ int mds_batch_destroy(mds_batch *b) {
         if (p) cudaFree(p);
     // chains other than a dataset's first do not own Y
     for (size_t g = 0; g < b->ctx.size(); ++g) mds_destroy(b->ctx[g]);
+    void *words[] = {b->scal_all, b->counters_all, b->err_all};
+    for (void *p : words)
+        if (p) cudaFree(p);
+    if (b->host) cudaFreeHost(b->host);
     if (b->cap_stream) cudaStreamDestroy(b->cap_stream);
     if (b->ev0) cudaEventDestroy(b->ev0);
     if (b->ev1) cudaEventDestroy(b->ev1);
@@ -3446,10 +3556,12 @@ int mds_batch_evaluate(mds_batch *b, double *loglik, double *dlogl_dsigma) {
     if (!b) return MDS_ERR_INVALID_ARG;
     BCU(cudaSetDevice(b->device));
     CHECK(batch_evaluate(b));
+    const size_t bytes = b->ctx.size() * kScalars * sizeof(double);
+    CHECK(batch_host(b, bytes));
+    BCU(cudaMemcpyAsync(b->host, b->scal_all, bytes, cudaMemcpyDeviceToHost, b->stream));
+    BCU(cudaStreamSynchronize(b->stream));
     for (size_t g = 0; g < b->ctx.size(); ++g) {
-        double s[kScalars];
-        BCU(cudaMemcpyAsync(s, b->ctx[g]->scal, sizeof(s), cudaMemcpyDeviceToHost, b->stream));
-        BCU(cudaStreamSynchronize(b->stream));
+        const double *s = static_cast<const double *>(b->host) + g * kScalars;
         if (loglik) loglik[g] = s[kLogLik];
         if (dlogl_dsigma) dlogl_dsigma[g] = s[kDSigma];
     }
@@ -3463,6 +3575,7 @@ int mds_batch_hmc(mds_batch *b, int n_iter, int n_steps, const double *eps, uint
     if (n_iter < 0 || n_steps < 0 || !eps) return bfail(b, MDS_ERR_INVALID_ARG, "need n_iter, n_steps >= 0 and eps");
     for (int i = 0; i < b->n_data; ++i)
         if (!std::isfinite(eps[i])) return bfail(b, MDS_ERR_INVALID_ARG, "eps[%d] is not finite", i);
+    b->eps.assign(eps, eps + b->n_data);
     bool valid = true;
     for (mds_ctx *c : b->ctx) valid = valid && c->grad_valid;
     if (!valid)
@@ -3497,19 +3610,12 @@ int mds_batch_hmc(mds_batch *b, int n_iter, int n_steps, const double *eps, uint
             ac[g] = make_accept_args(c, n_steps, 1, 1, seed, static_cast<uint32_t>(g), sg,
                                      b->acc_out + static_cast<size_t>(g) * n_iter,
                                      b->dh_out + static_cast<size_t>(g) * n_iter, n_iter);
-            BCU(cudaMemsetAsync(c->counters + kIterLocal, 0, sizeof(int64_t), b->stream));
         }
     }
-    std::vector<ReduceArgs> rc(total);
-    for (int dd = 0; dd < b->n_data; ++dd)
-        for (int k = 0; k < b->chains[dd]; ++k) {
-            const int g = b->chain0[dd] + k;
-            rc[g] = reduce_args(b->ctx[g], kModeEval, eps[dd]);
-        }
+    BCU(cudaMemset2DAsync(b->counters_all + kIterLocal, kCounters * sizeof(int64_t), 0, sizeof(int64_t), total,
+                          b->stream));
     BCU(cudaMemcpyAsync(b->tcfg, tc.data(), total * sizeof(TrajArgs), cudaMemcpyHostToDevice, b->stream));
     BCU(cudaMemcpyAsync(b->acfg, ac.data(), total * sizeof(AcceptArgs), cudaMemcpyHostToDevice, b->stream));
-    BCU(cudaMemcpyAsync(b->rcfg, rc.data(), total * sizeof(ReduceArgs), cudaMemcpyHostToDevice, b->stream));
-    BCU(cudaStreamSynchronize(b->stream));
     const auto key = std::make_tuple(b->gen, n_steps);
     if (!b->graph || key != b->graph_key || max_grid != b->max_start_grid || max_nd != b->max_nd) {
         if (b->graph) {
@@ -3540,13 +3646,18 @@ int mds_batch_hmc(mds_batch *b, int n_iter, int n_steps, const double *eps, uint
         b->max_nd = max_nd;
     }
     for (int t = 0; t < n_iter; ++t) BCU(cudaGraphLaunch(b->graph, b->stream));
-    int st = batch_check_errors(b, "batch hmc");
+    // one read-back: H1 - H0, decisions, error words
+    const size_t res = static_cast<size_t>(total) * n_iter;
+    CHECK(batch_host(b, res * (sizeof(double) + sizeof(int32_t)) + total * sizeof(unsigned)));
+    double *h = static_cast<double *>(b->host);
+    int32_t *a = reinterpret_cast<int32_t *>(h + res);
+    unsigned *words = reinterpret_cast<unsigned *>(a + res);
+    if (dh) BCU(cudaMemcpyAsync(h, b->dh_out, res * sizeof(double), cudaMemcpyDeviceToHost, b->stream));
+    if (accepted) BCU(cudaMemcpyAsync(a, b->acc_out, res * sizeof(int32_t), cudaMemcpyDeviceToHost, b->stream));
+    BCU(cudaMemcpyAsync(words, b->err_all, total * sizeof(unsigned), cudaMemcpyDeviceToHost, b->stream));
+    BCU(cudaStreamSynchronize(b->stream));
+    int st = batch_status(b, words, "batch hmc");
     if (accepted || dh) {
-        std::vector<int32_t> a(static_cast<size_t>(total) * n_iter);
-        std::vector<double> h(static_cast<size_t>(total) * n_iter);
-        BCU(cudaMemcpyAsync(a.data(), b->acc_out, a.size() * sizeof(int32_t), cudaMemcpyDeviceToHost, b->stream));
-        BCU(cudaMemcpyAsync(h.data(), b->dh_out, h.size() * sizeof(double), cudaMemcpyDeviceToHost, b->stream));
-        BCU(cudaStreamSynchronize(b->stream));
         for (int t = 0; t < n_iter; ++t)
             for (int g = 0; g < total; ++g) {
                 if (accepted) accepted[static_cast<size_t>(t) * total + g] = a[static_cast<size_t>(g) * n_iter + t];

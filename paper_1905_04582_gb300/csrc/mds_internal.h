@@ -296,6 +296,13 @@ struct XState {
     unsigned *xmax_bits;      // FP32C: running max |x| (float bits, atomicMax)
 };
 
+// What calls hand back to the host, in pinned memory that the device writes.
+struct HostPub {
+    unsigned err;             // error bits of the call
+    float xmax;               // max |x| of the locations just set
+    double scal[kScalars];
+};
+
 struct ReduceArgs {
     const void *row_part;
     const void *col_part;
@@ -552,7 +559,10 @@ cudaError_t launch_ingest(const IngestArgs &a, cudaStream_t s);
 // Locations in: src (N x D, f32/f64) -> the state x (zero padded to n_pad)
 // and, on the FP32C path, the split layouts (quantum from *split).
 cudaError_t launch_set_x(const void *src, bool src_f64, int64_t n, int64_t n_pad, int d, bool fp64, const XState &xs,
-                         unsigned *err, cudaStream_t s);
+                         unsigned *err, HostPub *pub, cudaStream_t s);
+// Error word and scalars into pinned memory, the gradient (pairs: float2 (hi, lo), else double) into dst.
+cudaError_t launch_publish(const void *src, bool pairs, void *dst, bool dst_f64, int64_t count, const unsigned *err,
+                           const double *scal, HostPub *pub, cudaStream_t s);
 // Recompute the split layouts of the FP32C path from x (after a quantum change).
 cudaError_t launch_resplit(const XState &xs, int64_t n_pad, int d, cudaStream_t s);
 // Re-pack the tile-packed Y for a new slot order: the pair at new slots

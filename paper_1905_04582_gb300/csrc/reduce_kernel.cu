@@ -966,29 +966,86 @@ __global__ void repack_kernel(const float *old_y, float *new_y, const int32_t *m
 // --------------------------------------------------------------- set x
 
 // Locations from the caller.  FP32C: the split quantum follows from max |x|
-// of the incoming values (xmax_kernel ran just before on the same stream);
-// every thread derives the same quantum by the host/device rule
-// (choose_split) and CTA 0 stores it.  Outside the FP32C range nothing is
-// written and the range bit is raised, so the previous state stays intact.
-template <typename T, typename S>
-__global__ void set_x_kernel(const S *src, int64_t n, int64_t n_pad, int d, XState xs, unsigned *err) {
+// of the incoming values; every CTA derives the same quantum by the
+// host/device rule (choose_split, one thread of it: the rule's FP64 division
+// by every warp took longer than the rest of the kernel) and CTA 0 stores it.
+// Outside the FP32C range nothing is written and the range bit is raised, so
+// the previous state stays intact.  The call's error bits go to `pub` (pinned
+// host memory: the host reads them after its wait, without a copy); bits that
+// earlier work left in the context's error word are cleared.
+//
+// ONE: each CTA finds max |x| by reading all of X itself (16-byte loads, at
+// most 16 a thread), which replaces a launch, two memsets and their hand-over;
+// up to kSetXOne elements.  Beyond, xmax_kernel runs just before.
+constexpr int kSetXThreads = 512;
+constexpr int64_t kSetXOne = 32768;
+
+template <typename S>
+__device__ __forceinline__ float abs_max(const S *src, int64_t count) {
+    constexpr int kV = 16 / sizeof(S);
+    struct alignas(16) Vec {
+        S v[kV];
+    };
+    float m = 0.f;
+    const int64_t vecs = (reinterpret_cast<uintptr_t>(src) & 15) == 0 ? count / kV : 0;
+#pragma unroll 8
+    for (int64_t e = threadIdx.x; e < vecs; e += kSetXThreads) {
+        const Vec w = reinterpret_cast<const Vec *>(src)[e];
+#pragma unroll
+        for (int i = 0; i < kV; ++i) m = fmaxf(m, fabsf(static_cast<float>(w.v[i])));
+    }
+#pragma unroll 8
+    for (int64_t e = vecs * kV + threadIdx.x; e < count; e += kSetXThreads)
+        m = fmaxf(m, fabsf(static_cast<float>(src[e])));
+    return m;
+}
+
+template <typename T, typename S, bool ONE>
+__global__ void __launch_bounds__(kSetXThreads)
+    set_x_kernel(const S *src, int64_t n, int64_t n_pad, int d, XState xs, unsigned *err, HostPub *pub) {
+    const bool first = blockIdx.x == 0 && threadIdx.x == 0;
     Split sp{};
     if constexpr (std::is_same<T, float>::value) {
-        if (!choose_split(__uint_as_float(*xs.xmax_bits), d, sp)) {
-            if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(err, kErrRange);
+        __shared__ float sm[kSetXThreads / 32];
+        __shared__ Split sp_s;
+        __shared__ int ok_s;
+        float m;
+        if constexpr (ONE)
+            m = block_max<kSetXThreads>(abs_max(src, n * d), sm);
+        else
+            m = __uint_as_float(*xs.xmax_bits);
+        if (threadIdx.x == 0) {
+            Split s1{};
+            ok_s = choose_split(m, d, s1);
+            sp_s = s1;
+        }
+        __syncthreads();
+        sp = sp_s;
+        if (first) {
+            pub->xmax = m;
+            *err = 0u;
+        }
+        if (!ok_s) {
+            if (first) atomicOr(&pub->err, kErrRange);
             return;
         }
-        if (blockIdx.x == 0 && threadIdx.x == 0) *xs.split = sp;
+        if (first) {
+            *xs.split = sp;
+            if constexpr (ONE) *xs.xmax_bits = __float_as_uint(m);
+        }
+    } else if (first) {
+        *err = 0u;
     }
     const int64_t total = n_pad * d;
-    for (int64_t e = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; e < total;
-         e += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+    bool bad = false;
+    for (int64_t e = static_cast<int64_t>(blockIdx.x) * kSetXThreads + threadIdx.x; e < total;
+         e += static_cast<int64_t>(gridDim.x) * kSetXThreads) {
         const int64_t k = e / d;
         const int kk = static_cast<int>(e % d);
         T v = T(0);
         if (k < n) {
-            const double sv = static_cast<double>(src[e]);
-            if (!isfinite(sv)) atomicOr(err, kErrBadInput);
+            const S sv = src[e];
+            bad = bad || !isfinite(sv);
             v = static_cast<T>(sv);
         }
         if constexpr (std::is_same<T, float>::value)
@@ -996,6 +1053,7 @@ __global__ void set_x_kernel(const S *src, int64_t n, int64_t n_pad, int d, XSta
         else
             store_x<T>(xs, k, d, kk, v);
     }
+    if (bad) atomicOr(&pub->err, kErrBadInput);
 }
 
 __global__ void resplit_kernel(XState xs, int64_t total, int d) {
@@ -1028,6 +1086,33 @@ __global__ void convert_kernel(const void *src, int kind, T *dst, int64_t count)
         else {
             const float2 g = reinterpret_cast<const float2 *>(src)[e];
             dst[e] = static_cast<T>(static_cast<double>(g.x) + static_cast<double>(g.y));
+        }
+    }
+}
+
+// The end of an evaluation: the gradient converted into the caller's buffer
+// (dst null: none), the error word and the scalars into pinned host memory, so
+// that one wait hands everything over (a copy each for the error word and the
+// scalars, the first with a wait of its own before the conversion could be
+// launched, took longer than the pass at small N).  With an error bit set the
+// caller's buffer stays as it was.
+template <typename T>
+__global__ void publish_kernel(const void *src, bool pairs, T *dst, int64_t count, const unsigned *err,
+                               const double *scal, HostPub *pub) {
+    pdl_wait();
+    const unsigned h = __ldcg(err);
+    if (blockIdx.x == 0) {
+        if (threadIdx.x < kScalars) pub->scal[threadIdx.x] = scal[threadIdx.x];
+        if (threadIdx.x == 0) pub->err = h;
+    }
+    if (h != 0u || !dst) return;
+    for (int64_t e = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; e < count;
+         e += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+        if (pairs) {
+            const float2 g = reinterpret_cast<const float2 *>(src)[e];
+            dst[e] = static_cast<T>(static_cast<double>(g.x) + static_cast<double>(g.y));
+        } else {
+            dst[e] = static_cast<T>(reinterpret_cast<const double *>(src)[e]);
         }
     }
 }
@@ -1151,20 +1236,42 @@ cudaError_t launch_ingest(const IngestArgs &a, cudaStream_t s) {
 }
 
 cudaError_t launch_set_x(const void *src, bool src_f64, int64_t n, int64_t n_pad, int d, bool fp64, const XState &xs,
-                         unsigned *err, cudaStream_t s) {
-    const int g = grid_for(n_pad * d, 256);
+                         unsigned *err, HostPub *pub, cudaStream_t s) {
+    const int g = grid_for(n_pad * d, kSetXThreads);
+    const bool one = n * d <= kSetXOne;
+    if (!fp64 && !one) {
+        cudaError_t e = cudaMemsetAsync(xs.xmax_bits, 0, sizeof(unsigned), s);
+        if (e == cudaSuccess) e = launch_xmax(src, src_f64, n * d, xs.xmax_bits, s);
+        if (e != cudaSuccess) return e;
+    }
+    const double *sd = static_cast<const double *>(src);
+    const float *sf = static_cast<const float *>(src);
     if (fp64) {
         if (src_f64)
-            set_x_kernel<double, double><<<g, 256, 0, s>>>(static_cast<const double *>(src), n, n_pad, d, xs, err);
+            set_x_kernel<double, double, false><<<g, kSetXThreads, 0, s>>>(sd, n, n_pad, d, xs, err, pub);
         else
-            set_x_kernel<double, float><<<g, 256, 0, s>>>(static_cast<const float *>(src), n, n_pad, d, xs, err);
+            set_x_kernel<double, float, false><<<g, kSetXThreads, 0, s>>>(sf, n, n_pad, d, xs, err, pub);
+    } else if (one) {
+        if (src_f64)
+            set_x_kernel<float, double, true><<<g, kSetXThreads, 0, s>>>(sd, n, n_pad, d, xs, err, pub);
+        else
+            set_x_kernel<float, float, true><<<g, kSetXThreads, 0, s>>>(sf, n, n_pad, d, xs, err, pub);
     } else {
         if (src_f64)
-            set_x_kernel<float, double><<<g, 256, 0, s>>>(static_cast<const double *>(src), n, n_pad, d, xs, err);
+            set_x_kernel<float, double, false><<<g, kSetXThreads, 0, s>>>(sd, n, n_pad, d, xs, err, pub);
         else
-            set_x_kernel<float, float><<<g, 256, 0, s>>>(static_cast<const float *>(src), n, n_pad, d, xs, err);
+            set_x_kernel<float, float, false><<<g, kSetXThreads, 0, s>>>(sf, n, n_pad, d, xs, err, pub);
     }
     return cudaGetLastError();
+}
+
+cudaError_t launch_publish(const void *src, bool pairs, void *dst, bool dst_f64, int64_t count, const unsigned *err,
+                           const double *scal, HostPub *pub, cudaStream_t s) {
+    const dim3 g(dst ? grid_for(count, 256) : 1), b(256);
+    cudaError_t e =
+        dst_f64 ? launch_pdl(publish_kernel<double>, g, b, 0, s, src, pairs, static_cast<double *>(dst), count, err, scal, pub)
+                : launch_pdl(publish_kernel<float>, g, b, 0, s, src, pairs, static_cast<float *>(dst), count, err, scal, pub);
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 cudaError_t launch_repack(const float *old_y, float *new_y, const int32_t *map, int64_t n, int32_t nt, cudaStream_t s) {

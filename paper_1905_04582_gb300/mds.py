@@ -564,7 +564,7 @@ if torch is not None:
             ctx.ds = ds
             ctx.x_dtype = x.dtype
             ctx.s_dtype = sigma.dtype
-            return torch.tensor(ll, dtype=torch.float64, device=x.device)
+            return torch.full((), ll, dtype=torch.float64, device=x.device)
 
         @staticmethod
         def backward(ctx, gout):
