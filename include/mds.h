@@ -542,10 +542,10 @@ int mds_batch_hmc(mds_batch *b, int n_iter, int n_steps, const double *eps, uint
 /* Shape of the batched pass.  strip in [1, 8]: the batched strip kernel,
  * strip tiles of one row block per CTA, each Y tile loaded into shared memory
  * once for all chains of its dataset.  strip in [-256, -1]: every chain's own
- * chunked pass (chunks of about -strip tiles), all chains' passes as
- * concurrent branches between the same reduction steps; Y is read once per
- * chain, from L2 where the datasets' Y fit.  0: autotune over both by timing
- * (strips of 1-4 tiles, chunks of 2-16 tiles).
+ * chunked pass (chunks of about -strip tiles), all chains' passes in one
+ * launch; Y is read once per chain, from L2 where the datasets' Y fit.
+ * 0: autotune over both by timing (strips of 1-4 tiles, chunks of 2-16 tiles
+ * or of one to three full waves).
  * mds_batch_get_strip returns the shape in use in the same encoding. */
 int mds_batch_set_strip(mds_batch *b, int32_t strip);
 /* Locality order for every dataset of a batch (as mds_reorder, section 2.5's

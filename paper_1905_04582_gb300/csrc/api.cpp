@@ -3060,8 +3060,6 @@ struct mds_batch {
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     int32_t strip = 0, strip_req = 0;  // > 0: the batched strip kernel; < 0: per-chain chunked passes
                                        // of about -strip tiles per chunk
-    cudaEvent_t fork = nullptr;        // per-chain passes: fork from the batch stream ...
-    std::vector<cudaEvent_t> joins;    // ... and join back, one event per chain
     BatchDataset *ds_dev = nullptr;
     BatchChain *ch_dev = nullptr;
     BatchStrip *strips_dev = nullptr;
@@ -3069,6 +3067,7 @@ struct mds_batch {
     int32_t n_strips = 0;
     ReduceArgs *rcfg = nullptr;
     int2 *jobs = nullptr;
+    int quarters = 0;          // CTAs per column block of the reduction
     size_t jobs_cap = 0;
     int32_t n_jobs = 0;
     TrajArgs *tcfg = nullptr;
@@ -3205,6 +3204,13 @@ int batch_tables(mds_batch *b, int strip) {
     std::vector<BatchStrip> st;
     std::vector<int2> jobs;
     std::vector<ReduceArgs> rc(total);
+    // whole column blocks where quarters of them would already be more than
+    // the resident CTAs (see reduce_batch_kernel)
+    int64_t blocks = 0;
+    for (const mds_ctx *c : b->ctx) blocks += c->nt;
+    const int quarters = blocks * kReduceQuarters > static_cast<int64_t>(b->sm_count) * kReduceResident ? 1 : kReduceQuarters;
+    if (quarters != b->quarters) b->gen++;
+    b->quarters = quarters;
     for (int dd = 0; dd < b->n_data; ++dd) {
         const mds_ctx *c0 = b->ctx[b->chain0[dd]];
         const PairArgs pa = pair_args(c0);
@@ -3233,7 +3239,7 @@ int batch_tables(mds_batch *b, int strip) {
         ch[g] = BatchChain{c->xrow, c->xcol, static_cast<float *>(c->row_part), static_cast<float *>(c->col_part),
                            static_cast<float *>(c->scal_part)};
         rc[g] = reduce_args(c, kModeEval, eps_of(b, g));
-        for (int J = 0; J < c->nt * kReduceQuarters; ++J) jobs.push_back(make_int2(g, J));
+        for (int J = 0; J < c->nt * quarters; ++J) jobs.push_back(make_int2(g, J));
         jobs.push_back(make_int2(g, -1));
     }
     if (st.size() > b->strips_cap) {
@@ -3284,21 +3290,26 @@ BatchPairArgs batch_pair_args(const mds_batch *b) {
 int batch_enqueue_pass(mds_batch *b, int mode, cudaStream_t s) {
     cudaError_t e = cudaSuccess;
     if (b->strip < 0) {
-        // every chain's chunked pass on its own stream (graph branches when
-        // captured), all after the work before on s, all before the reduction
-        e = cudaEventRecord(b->fork, s);
-        for (size_t g = 0; e == cudaSuccess && g < b->ctx.size(); ++g) {
-            mds_ctx *c = b->ctx[g];
-            e = cudaStreamWaitEvent(c->cap_stream, b->fork, 0);
-            if (e == cudaSuccess) e = launch_pair_chunks_f32(pair_args(c), static_cast<int>(b->d), c->cap_stream, false, 0);
-            if (e == cudaSuccess) e = cudaEventRecord(b->joins[g], c->cap_stream);
+        // every chain's chunked pass, kChunkBatch chains to a launch
+        ChunkBatchArgs a{};
+        const size_t total = b->ctx.size();
+        for (size_t g0 = 0; e == cudaSuccess && g0 < total; g0 += kChunkBatch) {
+            a.n_chains = static_cast<int32_t>(std::min<size_t>(kChunkBatch, total - g0));
+            a.first[0] = 0;
+            bool long_runs = false;
+            for (int k = 0; k < a.n_chains; ++k) {
+                const mds_ctx *c = b->ctx[g0 + k];
+                a.chain[k] = pair_args(c);
+                a.first[k + 1] = a.first[k] + a.chain[k].n_strips;
+                long_runs = long_runs || c->chunk_long_runs;
+            }
+            e = launch_pair_chunks_batch(a, static_cast<int>(b->d), long_runs, s);
         }
-        for (size_t g = 0; e == cudaSuccess && g < b->ctx.size(); ++g) e = cudaStreamWaitEvent(s, b->joins[g], 0);
     } else {
         e = launch_pair_batch(batch_pair_args(b), b->d, b->grid, s);
     }
     if (e != cudaSuccess) return bfail(b, MDS_ERR_CUDA, "batched pair pass: %s", cudaGetErrorString(e));
-    e = launch_reduce_batch(b->rcfg, b->jobs, b->n_jobs, b->d, mode, s);
+    e = launch_reduce_batch(b->rcfg, b->jobs, b->n_jobs, b->d, mode, b->quarters, s);
     if (e != cudaSuccess) return bfail(b, MDS_ERR_CUDA, "batched reduction: %s", cudaGetErrorString(e));
     return MDS_OK;
 }
@@ -3339,10 +3350,23 @@ int batch_autotune(mds_batch *b) {
         }
         if (s == 0) {
             float best_ms = 1e30f;
+            // the strip kernel, chunks of a few tiles, and chunks that make one,
+            // two or three full waves of the resident chunk slots
+            std::vector<int> cands = {1, 2, 3, 4, -2, -4, -8, -16};
+            const int64_t slots = static_cast<int64_t>(b->sm_count) * std::max(1, pair_chunk_blocks_per_sm(b->d));
+            for (int m : {1, 2, 3}) {
+                int per = 1;
+                auto chunks = [&] {
+                    int64_t k = 0;
+                    for (const mds_ctx *c : b->ctx) k += std::max<int64_t>(1, c->tiles / per);
+                    return k;
+                };
+                while (per < 256 && chunks() > slots * m) ++per;
+                if (std::find(cands.begin(), cands.end(), -per) == cands.end()) cands.push_back(-per);
+            }
             // each candidate timed as the HMC runs it: a captured graph of
-            // five passes with their reductions (the per-chain shapes launch
-            // one kernel per chain, which eager launches would slow)
-            for (int cand : {1, 2, 3, 4, -2, -4, -6, -8, -16}) {
+            // five passes with their reductions
+            for (int cand : cands) {
                 if (cand > 0 && pair_batch_blocks_per_sm(b->d, cand) <= 0) continue;
                 CHECK(batch_tables(b, cand));
                 CHECK(batch_enqueue_pass(b, kModeEval, b->stream));
@@ -3443,8 +3467,7 @@ int mds_batch_create(int32_t n_data, const int64_t *n, int32_t d, const int32_t 
     if ((st = bdev_alloc(b, &b->tcfg, total * sizeof(TrajArgs)))) return cleanup(st);
     if ((st = bdev_alloc(b, &b->acfg, total * sizeof(AcceptArgs)))) return cleanup(st);
     bool ev_ok = cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking) == cudaSuccess &&
-                 cudaEventCreate(&b->ev0) == cudaSuccess && cudaEventCreate(&b->ev1) == cudaSuccess &&
-                 cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming) == cudaSuccess;
+                 cudaEventCreate(&b->ev0) == cudaSuccess && cudaEventCreate(&b->ev1) == cudaSuccess;
     if ((st = bdev_alloc(b, &b->scal_all, static_cast<size_t>(total) * kScalars * sizeof(double)))) return cleanup(st);
     if ((st = bdev_alloc(b, &b->counters_all, static_cast<size_t>(total) * kCounters * sizeof(int64_t))))
         return cleanup(st);
@@ -3466,9 +3489,6 @@ int mds_batch_create(int32_t n_data, const int64_t *n, int32_t d, const int32_t 
         x->err = b->err_all + g;
         x->shared_words = true;
     }
-    b->joins.assign(b->ctx.size(), nullptr);
-    for (size_t g = 0; ev_ok && g < b->ctx.size(); ++g)
-        ev_ok = cudaEventCreateWithFlags(&b->joins[g], cudaEventDisableTiming) == cudaSuccess;
     if (!ev_ok) {
         b->last_error = "stream/event creation failed";
         return cleanup(MDS_ERR_CUDA);
@@ -3494,9 +3514,6 @@ int mds_batch_destroy(mds_batch *b) {
     if (b->cap_stream) cudaStreamDestroy(b->cap_stream);
     if (b->ev0) cudaEventDestroy(b->ev0);
     if (b->ev1) cudaEventDestroy(b->ev1);
-    if (b->fork) cudaEventDestroy(b->fork);
-    for (cudaEvent_t e : b->joins)
-        if (e) cudaEventDestroy(e);
     delete b;
     return MDS_OK;
 }
@@ -3610,6 +3627,7 @@ int mds_batch_hmc(mds_batch *b, int n_iter, int n_steps, const double *eps, uint
             ac[g] = make_accept_args(c, n_steps, 1, 1, seed, static_cast<uint32_t>(g), sg,
                                      b->acc_out + static_cast<size_t>(g) * n_iter,
                                      b->dh_out + static_cast<size_t>(g) * n_iter, n_iter);
+            if (n_steps > 0) ac[g].n_end_parts = static_cast<int32_t>(c->nt * b->quarters);
         }
     }
     BCU(cudaMemset2DAsync(b->counters_all + kIterLocal, kCounters * sizeof(int64_t), 0, sizeof(int64_t), total,

@@ -170,6 +170,17 @@ struct PairArgs {
     double inv_s2;
 };
 
+// One launch of several chains' chunked passes: chain g's chunks are the CTAs
+// [first[g], first[g + 1]).  A kernel argument (its limit is 32,764 bytes), so
+// that the arguments stay in constant memory as the single pass's do.
+constexpr int kChunkBatch = 64;
+struct ChunkBatchArgs {
+    int32_t n_chains;
+    int32_t first[kChunkBatch + 1];
+    PairArgs chain[kChunkBatch];
+};
+static_assert(sizeof(ChunkBatchArgs) <= 32764, "kernel argument size");
+
 enum ErrBits : unsigned {
     kErrTimeout = 1u,     // a bounded mbarrier wait gave up
     kErrNonfinite = 2u,   // a partial sum was NaN / Inf
@@ -239,6 +250,7 @@ cudaError_t launch_pair_pass_f32(const PairArgs &a, int d, cudaStream_t s, bool 
 // one CTA each.
 // grouped: one CTA per SM whose groups of four warps each run a chunk
 // (pair_chunk_groups(d) groups); otherwise one chunk per CTA.
+cudaError_t launch_pair_chunks_batch(const ChunkBatchArgs &b, int d, bool long_runs, cudaStream_t s);
 cudaError_t launch_pair_chunks_f32(const PairArgs &a, int d, cudaStream_t s, bool pdl = true, int smem_min = 0,
                                    bool grouped = false);
 int pair_chunk_smem_bytes(int d);
@@ -343,6 +355,7 @@ struct ReduceArgs {
 // The reduction runs kReduceQuarters CTAs per column block (16 items each)
 // plus one CTA for the scalars.
 constexpr int kReduceQuarters = 4;
+constexpr int kReduceResident = 4;  // CTAs per SM that the batched reduction is compiled for
 cudaError_t launch_reduce(const ReduceArgs &a, cudaStream_t s);
 
 // Trajectory start: (optionally) draw / load p, save x0 and the cached
@@ -408,7 +421,8 @@ cudaError_t launch_sigma_draws(uint64_t seed, uint32_t chain, int64_t iter0, int
 
 // Batched launches (one per step for all problems): per-problem argument
 // tables in device memory.  jobs[k] = (problem, column block J or -1).
-cudaError_t launch_reduce_batch(const ReduceArgs *cfg, const int2 *jobs, int n_jobs, int d, int mode, cudaStream_t s);
+cudaError_t launch_reduce_batch(const ReduceArgs *cfg, const int2 *jobs, int n_jobs, int d, int mode, int quarters,
+                                cudaStream_t s);
 int traj_start_grid(int64_t n, int d);
 cudaError_t launch_traj_start_batch(const TrajArgs *cfg, int n_chains, int max_grid, int d, cudaStream_t s);
 cudaError_t launch_traj_end_batch(const AcceptArgs *cfg, int n_chains, int64_t max_nd, int d, cudaStream_t s);

@@ -33,10 +33,8 @@ namespace {
 // reduction is launched as a programmatic dependent), and one round of loads
 // covers the partials of a block at N = 5392.
 constexpr int kRedThreads = 256;
-constexpr int kRedRows = 16;                       // items per CTA
 constexpr int kRedQuarters = kReduceQuarters;      // CTAs per column block
-static_assert(kRedQuarters * kRedRows == kTile, "quarters must cover a block");
-constexpr int kSplits = kRedThreads / kRedRows;
+constexpr int kRedRows = kTile / kRedQuarters;     // items per CTA
 constexpr double kLn2 = 0.69314718055994530942;
 constexpr double kSqrt2Pi = 2.50662827463100050242;
 
@@ -195,12 +193,15 @@ __device__ __forceinline__ void load_coords(const T *p, bool ok, T (&v)[D]) {
     }
 }
 
-template <typename T, int D>
+// ROWS items per CTA (kRedRows or a whole block), Jq counting CTAs.
+template <typename T, int D, int ROWS>
 __device__ __forceinline__ void reduce_body(const ReduceArgs &a, int mode, int Jq) {
+    constexpr int kRows = ROWS, kPerBlock = kTile / ROWS, kSplits = kRedThreads / ROWS;
+    static_assert(ROWS == 16 || ROWS == kTile, "combine of the splits");
     constexpr bool kF32 = std::is_same<T, float>::value;
     using Acc = typename std::conditional<kF32, DF, double>::type;
     using G = typename GradT<T>::type;
-    __shared__ Acc sm[kSplits * kRedRows > 64 ? kSplits * kRedRows : 64];
+    __shared__ Acc sm[64];
     const int tid = threadIdx.x;
     const int nt = a.nt;
     // the item at this thread's slot (the order is constant between passes,
@@ -208,11 +209,11 @@ __device__ __forceinline__ void reduce_body(const ReduceArgs &a, int mode, int J
     int64_t item_of_slot = -1;
     int s0 = 0, s1 = 0;  // the column block's row-partial slots (fixed between passes too)
     if (Jq >= 0) {
-        const int64_t ks = static_cast<int64_t>(Jq / kRedQuarters) * kTile + (Jq % kRedQuarters) * kRedRows +
-                           (tid % kRedRows);
+        const int64_t ks = static_cast<int64_t>(Jq / kPerBlock) * kTile + (Jq % kPerBlock) * kRows +
+                           (tid % kRows);
         item_of_slot = (a.perm && ks < a.n) ? a.perm[ks] : ks;
-        s0 = a.row_first_slot[Jq / kRedQuarters];
-        s1 = a.row_first_slot[Jq / kRedQuarters + 1];
+        s0 = a.row_first_slot[Jq / kPerBlock];
+        s1 = a.row_first_slot[Jq / kPerBlock + 1];
     }
     // the split quantum changes only at a trajectory's end (never in a
     // kick-drift launch): read before the wait, so that writing the split
@@ -345,9 +346,9 @@ __device__ __forceinline__ void reduce_body(const ReduceArgs &a, int mode, int J
         return;
     }
 
-    const int J = Jq / kRedQuarters;
-    const int r = (Jq % kRedQuarters) * kRedRows + (tid % kRedRows);  // row within the block
-    const int s = tid / kRedRows;
+    const int J = Jq / kPerBlock;
+    const int r = (Jq % kPerBlock) * kRows + (tid % kRows);  // row within the block
+    const int s = tid / kRows;
     const int64_t k = static_cast<int64_t>(J) * kTile + r;
     Acc acc[D];
 #pragma unroll
@@ -399,20 +400,25 @@ __device__ __forceinline__ void reduce_body(const ReduceArgs &a, int mode, int J
             }
     }
     // the kSplits partial sums of every (row, coordinate), in a fixed order:
-    // the two splits of a warp (lanes r and r + 16) by a shuffle, then the
-    // warps' sums through shared memory, all coordinates at once
-    constexpr int kRedWarps = kRedThreads / 32;
-    __shared__ Acc smw[kRedWarps * kRedRows * D];
+    // with 16 rows the two splits of a warp (lanes r and r + 16) by a shuffle
+    // first, then all through shared memory, all coordinates at once
+    constexpr int kParts = kRows == 16 ? kRedThreads / 32 : kSplits;
+    __shared__ Acc smw[kParts * kRows * D];
+    if constexpr (kRows == 16) {
 #pragma unroll
-    for (int d = 0; d < D; ++d) {
-        if constexpr (kF32)
-            df_add(acc[d], df_shfl_xor(acc[d], 16));
-        else
-            acc[d] += __shfl_xor_sync(0xffffffffu, acc[d], 16);
-    }
-    if ((tid & 31) < kRedRows) {
+        for (int d = 0; d < D; ++d) {
+            if constexpr (kF32)
+                df_add(acc[d], df_shfl_xor(acc[d], 16));
+            else
+                acc[d] += __shfl_xor_sync(0xffffffffu, acc[d], 16);
+        }
+        if ((tid & 31) < kRows) {
 #pragma unroll
-        for (int d = 0; d < D; ++d) smw[((tid >> 5) * kRedRows + (tid & 31)) * D + d] = acc[d];
+            for (int d = 0; d < D; ++d) smw[((tid >> 5) * kRows + (tid & 31)) * D + d] = acc[d];
+        }
+    } else {
+#pragma unroll
+        for (int d = 0; d < D; ++d) smw[tid * D + d] = acc[d];
     }
     __syncthreads();
     Acc gsum[D];
@@ -421,11 +427,11 @@ __device__ __forceinline__ void reduce_body(const ReduceArgs &a, int mode, int J
         for (int d = 0; d < D; ++d) {
             Acc g = smw[tid * D + d];
 #pragma unroll
-            for (int w = 1; w < kRedWarps; ++w) {
+            for (int w = 1; w < kParts; ++w) {
                 if constexpr (kF32)
-                    df_add(g, smw[(w * kRedRows + tid) * D + d]);
+                    df_add(g, smw[(w * kRows + tid) * D + d]);
                 else
-                    g += smw[(w * kRedRows + tid) * D + d];
+                    g += smw[(w * kRows + tid) * D + d];
             }
             gsum[d] = g;
         }
@@ -522,15 +528,20 @@ template <typename T, int D>
 __global__ void __launch_bounds__(kRedThreads) reduce_kernel(const __grid_constant__ ReduceArgs a) {
     const int last = a.nt * kRedQuarters;
     const int b = static_cast<int>(blockIdx.x);
-    reduce_body<T, D>(a, a.mode, b == last ? -1 : last - 1 - b);
+    reduce_body<T, D, kRedRows>(a, a.mode, b == last ? -1 : last - 1 - b);
 }
 
-// Batched: job (problem index, quarter-block index J * kReduceQuarters + q,
-// or -1 for the scalars) per CTA.
-template <int D>
-__global__ void __launch_bounds__(kRedThreads) reduce_batch_kernel(const ReduceArgs *cfg, const int2 *jobs, int mode) {
+// Batched: job (problem index, CTA of its column blocks, or -1 for the
+// scalars) per CTA.  ROWS = 64: a CTA per column block.  A CTA's time is a
+// chain of latencies (job, arguments, partials, state), so quarter blocks
+// cost when there are more of them than resident CTAs (2784 quarters on 152
+// SMs took 24 us of ncu's cold time for the 32 chains above; 728 blocks are
+// about one wave).
+template <int D, int ROWS>
+__global__ void __launch_bounds__(kRedThreads, D <= 4 ? kReduceResident : 2)
+    reduce_batch_kernel(const ReduceArgs *cfg, const int2 *jobs, int mode) {
     const int2 job = jobs[blockIdx.x];
-    reduce_body<float, D>(cfg[job.x], mode, job.y);
+    reduce_body<float, D, ROWS>(cfg[job.x], mode, job.y);
 }
 
 // ----------------------------------------------------------- traj start
@@ -1176,13 +1187,18 @@ cudaError_t launch_traj_end(const AcceptArgs &a, cudaStream_t s) {
         default: return cudaErrorInvalidValue;                                   \
     }
 
-cudaError_t launch_reduce_batch(const ReduceArgs *cfg, const int2 *jobs, int n_jobs, int d, int mode, cudaStream_t s) {
+cudaError_t launch_reduce_batch(const ReduceArgs *cfg, const int2 *jobs, int n_jobs, int d, int mode, int quarters,
+                                cudaStream_t s) {
     if (n_jobs <= 0) return cudaSuccess;
     // under PDL after the batched pass (reduce_body waits for it)
     cudaError_t e = cudaSuccess;
     switch (d) {
 #define MDS_RB_CASE(DD) \
-    case DD: e = launch_pdl(reduce_batch_kernel<DD>, dim3(n_jobs), dim3(kRedThreads), 0, s, cfg, jobs, mode); break;
+    case DD:                                                                                                        \
+        e = quarters == 1                                                                                           \
+                ? launch_pdl(reduce_batch_kernel<DD, kTile>, dim3(n_jobs), dim3(kRedThreads), 0, s, cfg, jobs, mode) \
+                : launch_pdl(reduce_batch_kernel<DD, kRedRows>, dim3(n_jobs), dim3(kRedThreads), 0, s, cfg, jobs, mode); \
+        break;
         MDS_RB_CASE(1) MDS_RB_CASE(2) MDS_RB_CASE(3) MDS_RB_CASE(4)
         MDS_RB_CASE(5) MDS_RB_CASE(6) MDS_RB_CASE(7) MDS_RB_CASE(8)
 #undef MDS_RB_CASE
