@@ -21,8 +21,8 @@ LIBDIR = os.path.join(HERE, "_lib")
 LIB = os.path.join(LIBDIR, "libmds.so")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-SOURCES = ["pair_kernel.cu", "chunk_kernel.cu", "batch_kernel.cu", "reduce_kernel.cu", "heldout.cu", "noalloc.cu", "tree_prior.cu", "rwmh.cu", "ceiling.cu", "tree_plan.cpp", "api.cpp"]
-HEADERS = ["mds_internal.h", "mills_ratio_coeffs.h", "pair_math.cuh", "pair_math64.cuh", "phi_table.h", "philox.cuh",
+SOURCES = ["pair_kernel.cu", "chunk_kernel.cu", "small_traj.cu", "batch_kernel.cu", "reduce_kernel.cu", "heldout.cu", "noalloc.cu", "tree_prior.cu", "rwmh.cu", "ceiling.cu", "tree_plan.cpp", "api.cpp"]
+HEADERS = ["chunk_tile.cuh", "df.cuh", "mds_internal.h", "mills_ratio_coeffs.h", "pair_math.cuh", "pair_math64.cuh", "phi_table.h", "philox.cuh",
            "tree_plan.h"]
 
 

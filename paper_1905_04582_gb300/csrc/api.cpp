@@ -97,6 +97,7 @@ struct mds_ctx {
                                   // bits come back with the next HMC read-back)
     uint64_t gen = 1;         // bumps whenever captured kernel arguments would change
     int start_grid = 0;
+    int small_fits = -1;      // small_traj_fits (device and size do not change), -1: not asked yet
 
     // device buffers
     float *y = nullptr;
@@ -1266,6 +1267,17 @@ AcceptArgs make_accept_args(const mds_ctx *c, int n_steps, int metropolis, int u
     return a;
 }
 
+// Whether trajectories run their steps in one launch: small FP32C problems
+// whose target is the likelihood with the isotropic prior, unless a shape of
+// the pass is forced or its passes are timed one by one.
+bool small_traj(mds_ctx *c) {
+    if (c->fp64 || c->tree_on || sharded(c) || c->profiling || c->stamping || c->strip_req > 0 || c->chunk_req != 0 ||
+        getenv("MDS_STRIP") || getenv("MDS_CHUNKS"))
+        return false;
+    if (c->small_fits < 0) c->small_fits = small_traj_fits(c->nt, c->d) ? 1 : 0;
+    return c->small_fits == 1;
+}
+
 // Enqueue one trajectory: start kernel, n_steps fused pair passes with their
 // leapfrog updates, end kernel (Metropolis when metropolis != 0).
 int enqueue_trajectory(mds_ctx *c, int n_steps, double eps, int momentum_src, int u_src, int metropolis,
@@ -1275,7 +1287,22 @@ int enqueue_trajectory(mds_ctx *c, int n_steps, double eps, int momentum_src, in
     cudaError_t e = launch_traj_start(t, &grid, s);
     if (e != cudaSuccess) return fail(c, MDS_ERR_CUDA, "trajectory start: %s", cudaGetErrorString(e));
     c->start_grid = grid;
-    for (int k = 0; k < n_steps; ++k)
+    int k0 = 0;
+    if (n_steps > 1 && small_traj(c)) {
+        // all steps but the last (which gives the end's energies) in one launch
+        k0 = n_steps - 1;
+        SmallTrajArgs st{};
+        st.pair = pair_args(c);
+        st.pair.xcol2 = c->xcol2;
+        st.reduce = reduce_args(c, kModeKickDrift, eps);
+        const double scale = -1.0 / (c->sigma * c->sigma);
+        const float h = static_cast<float>(scale);
+        st.reduce.part_scale_df = make_float2(h, static_cast<float>(scale - static_cast<double>(h)));
+        st.n_steps = k0;
+        e = launch_small_traj(st, c->d, s);
+        if (e != cudaSuccess) return fail(c, MDS_ERR_CUDA, "trajectory steps: %s", cudaGetErrorString(e));
+    }
+    for (int k = k0; k < n_steps; ++k)
         CHECK(enqueue_pass(c, k + 1 < n_steps ? kModeKickDrift : kModeHalfKick, eps, s));
     AcceptArgs a = make_accept_args(c, n_steps, metropolis, u_src, seed, 0, grid, c->acc_out, c->dh_out,
                                     static_cast<int64_t>(c->out_cap));

@@ -352,6 +352,15 @@ struct ReduceArgs {
     unsigned *err;
 };
 
+// Kick-drift steps of a small problem in one launch (small_traj.cu).
+constexpr int kStMaxBlocks = 7;            // row blocks at most
+constexpr int kStMaxSmem = 224 * 1024;     // shared memory of a CTA at most
+struct SmallTrajArgs {
+    PairArgs pair;
+    ReduceArgs reduce;        // mode kModeKickDrift, part_scale_df -1/sigma^2
+    int32_t n_steps;
+};
+
 // The reduction runs kReduceQuarters CTAs per column block (16 items each)
 // plus one CTA for the scalars.
 constexpr int kReduceQuarters = 4;
@@ -572,6 +581,8 @@ cudaError_t launch_ingest(const IngestArgs &a, cudaStream_t s);
 
 // Locations in: src (N x D, f32/f64) -> the state x (zero padded to n_pad)
 // and, on the FP32C path, the split layouts (quantum from *split).
+bool small_traj_fits(int64_t nt, int d);
+cudaError_t launch_small_traj(const SmallTrajArgs &a, int d, cudaStream_t s);
 cudaError_t launch_set_x(const void *src, bool src_f64, int64_t n, int64_t n_pad, int d, bool fp64, const XState &xs,
                          unsigned *err, HostPub *pub, cudaStream_t s);
 // Error word and scalars into pinned memory, the gradient (pairs: float2 (hi, lo), else double) into dst.
