@@ -797,6 +797,11 @@ int harvest_prof(mds_ctx *c) {
     return MDS_OK;
 }
 
+// CTAs of the tree prior's traversal (0: no tree prior).
+int tree_ctas(const mds_ctx *c) {
+    return c->tree_on ? (c->tree.n_trees + (c->tree.n_lone > 0 ? 1 : 0)) * c->tree.cluster : 0;
+}
+
 int enqueue_pass(mds_ctx *c, int mode, double eps, cudaStream_t s, bool plant_nan = false) {
     PairArgs a = pair_args(c);
     const int pk = c->prof_used;
@@ -826,19 +831,23 @@ int enqueue_pass(mds_ctx *c, int mode, double eps, cudaStream_t s, bool plant_na
         if (e != cudaSuccess) return fail(c, MDS_ERR_CUDA, "tree prior launch: %s", cudaGetErrorString(e));
     }
     // With a tree prior, launched early by PDL the pass's CTAs would hold
-    // every SM before the traversal's clusters could be placed.  So either
-    // the FP32C pass keeps PDL with its shared memory padded to leave room
-    // for one traversal CTA beside three pass CTAs on every SM (tree_pass_smem,
-    // chosen when the tree prior is set), or it is launched without PDL and
-    // becomes eligible when the traversal does.
-    const bool capped = c->tree_on && !c->fp64 && c->tree_pass_smem > 0;
+    // every SM before the traversal's clusters could be placed.  So the strip
+    // pass keeps PDL with its shared memory padded to leave room for one
+    // traversal CTA beside three pass CTAs on every SM (tree_pass_smem, chosen
+    // when the tree prior is set); any other pass is launched without PDL and
+    // becomes eligible when the traversal does.  The chunked pass's three CTAs
+    // of 168 registers fill an SM's register file whatever their shared
+    // memory: under PDL the traversal ran after it (47 us a step at N = 5392
+    // for a pass of 27 and a traversal of 22), so the tuner times the shapes
+    // with the traversal (TuneKey::tree): strips of 2 there, 31 us.
+    const bool capped = c->tree_on && !c->fp64 && c->pass_kind != kPassChunks && c->tree_pass_smem > 0;
     const bool pdl = !c->tree_on || capped;
     if (c->fp64)
         e = launch_pair_pass_f64(a, c->d, s, pdl);
     else if (c->pass_kind == kPassChunks)
         // the grouped form leaves no room for a traversal CTA: with a tree
         // prior the same chunks run one per CTA
-        e = launch_pair_chunks_f32(a, c->d, s, pdl, capped ? c->tree_pass_smem : 0, c->chunk_grouped && !c->tree_on);
+        e = launch_pair_chunks_f32(a, c->d, s, pdl, c->chunk_grouped && !c->tree_on);
     else
         e = launch_pair_pass_f32(a, c->d, s, pdl, capped ? c->tree_pass_smem : 0);
     if (e != cudaSuccess) return fail(c, MDS_ERR_CUDA, "pair pass launch: %s", cudaGetErrorString(e));
@@ -904,8 +913,9 @@ struct TuneKey {
     int d;
     bool fp64;
     bool reordered;
+    int tree;  // CTAs of a tree prior's traversal beside the pass (0: none): they take slots of the pass's
     bool operator<(const TuneKey &o) const {
-        return std::tie(gpu, n, d, fp64, reordered) < std::tie(o.gpu, o.n, o.d, o.fp64, o.reordered);
+        return std::tie(gpu, n, d, fp64, reordered, tree) < std::tie(o.gpu, o.n, o.d, o.fp64, o.reordered, o.tree);
     }
 };
 struct TuneVal {
@@ -951,7 +961,10 @@ void tune_load() {
         }
         fld.push_back(cur);
         if (fld.size() != 8) continue;
-        TuneKey k{fld[0], atoll(fld[1].c_str()), atoi(fld[2].c_str()), fld[3] == "fp64", fld[4] == "locality"};
+        const size_t plus = fld[4].find("+tree");
+        const int tree = plus == std::string::npos ? 0 : atoi(fld[4].c_str() + plus + 5);
+        TuneKey k{fld[0], atoll(fld[1].c_str()), atoi(fld[2].c_str()), fld[3] == "fp64",
+                  fld[4].substr(0, plus) == "locality", tree};
         TuneVal v{atoi(fld[5].c_str()), atoi(fld[6].c_str()), atof(fld[7].c_str())};
         // chunked: param chunks per slot (1..8), or for kPassChunks minus an
         // exact chunk count
@@ -971,9 +984,10 @@ void tune_save() {
     FILE *f = fopen(tmp.c_str(), "w");
     if (!f) return;
     for (const auto &kv : g_tune_cache)
-        fprintf(f, "%s\t%lld\t%d\t%s\t%s\t%d\t%d\t%.6f\n", kv.first.gpu.c_str(), static_cast<long long>(kv.first.n),
+        fprintf(f, "%s\t%lld\t%d\t%s\t%s%s\t%d\t%d\t%.6f\n", kv.first.gpu.c_str(), static_cast<long long>(kv.first.n),
                 kv.first.d, kv.first.fp64 ? "fp64" : "fp32c", kv.first.reordered ? "locality" : "caller",
-                kv.second.kind, kv.second.param, kv.second.ms);
+                kv.first.tree > 0 ? ("+tree" + std::to_string(kv.first.tree)).c_str() : "", kv.second.kind,
+                kv.second.param, kv.second.ms);
     const bool ok = fclose(f) == 0;
     if (ok) rename(tmp.c_str(), path.c_str());
     else remove(tmp.c_str());
@@ -1029,7 +1043,8 @@ int autotune(mds_ctx *c) {
         const int m = atoi(env);
         if (m > 0 && !c->fp64) return apply_shape(c, kPassChunks, std::min(m, 8));
     }
-    const TuneKey key{c->device_name, c->n, static_cast<int>(c->d), c->fp64, c->reordered};
+    const TuneKey key{c->device_name, c->n, static_cast<int>(c->d), c->fp64, c->reordered,
+                      tree_ctas(c)};
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
         tune_load();
@@ -1067,6 +1082,12 @@ int autotune(mds_ctx *c) {
         const int64_t uncut = (c->tiles * 5 + 4 * cut - 1) / (4 * cut);
         if (uncut > static_cast<int64_t>(c->sm_count) * per_sm * 6 && uncut <= (1 << 26))
             cands.emplace_back(kPassChunks, -static_cast<int>(uncut));
+        // slots left free for a tree prior's traversal, one CTA or two a slot
+        const int64_t slots = static_cast<int64_t>(c->sm_count) * per_sm;
+        for (int k : {1, 2}) {
+            const int64_t left = slots - (tree_ctas(c) + k - 1) / k;
+            if (c->tree_on && 2 * left >= slots && left <= c->tiles) cands.emplace_back(kPassChunks, -static_cast<int>(left));
+        }
         // the grouped form (not beside a tree prior's traversal, which it
         // leaves no room for)
         const int per_sm_g = pair_chunk_blocks_per_sm(c->d, true);

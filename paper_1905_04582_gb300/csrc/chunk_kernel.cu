@@ -442,15 +442,14 @@ cudaError_t launch_cap(const PairArgs &a, cudaStream_t s, bool pdl, int smem) {
 }
 
 template <int D>
-cudaError_t launch_d(const PairArgs &a, cudaStream_t s, bool pdl, int smem_min, bool grouped) {
+cudaError_t launch_d(const PairArgs &a, cudaStream_t s, bool pdl, bool grouped) {
     constexpr int G = chunk_slots_per_sm<D>();
     if (grouped && !a.tile_ho) {
         // held-out passes keep the one-group form (the chunk table serves both:
         // the same chunk slots per SM)
-        const int smem = smem_min > chunk_cta_smem<D, G>() ? smem_min : chunk_cta_smem<D, G>();
-        return launch_cap<D, false, G>(a, s, pdl, smem);
+        return launch_cap<D, false, G>(a, s, pdl, chunk_cta_smem<D, G>());
     }
-    const int smem = smem_min > chunk_cta_smem<D, 1>() ? smem_min : chunk_cta_smem<D, 1>();
+    constexpr int smem = chunk_cta_smem<D, 1>();
     return a.tile_ho ? launch_cap<D, true, 1>(a, s, pdl, smem) : launch_cap<D, false, 1>(a, s, pdl, smem);
 }
 
@@ -520,16 +519,16 @@ int pair_chunk_blocks_per_sm(int d, bool grouped) {
 
 int pair_chunk_groups(int d) { return d <= 4 ? chunk_slots_per_sm<1>() : chunk_slots_per_sm<8>(); }
 
-cudaError_t launch_pair_chunks_f32(const PairArgs &a, int d, cudaStream_t s, bool pdl, int smem_min, bool grouped) {
+cudaError_t launch_pair_chunks_f32(const PairArgs &a, int d, cudaStream_t s, bool pdl, bool grouped) {
     switch (d) {
-        case 1: return launch_d<1>(a, s, pdl, smem_min, grouped);
-        case 2: return launch_d<2>(a, s, pdl, smem_min, grouped);
-        case 3: return launch_d<3>(a, s, pdl, smem_min, grouped);
-        case 4: return launch_d<4>(a, s, pdl, smem_min, grouped);
-        case 5: return launch_d<5>(a, s, pdl, smem_min, grouped);
-        case 6: return launch_d<6>(a, s, pdl, smem_min, grouped);
-        case 7: return launch_d<7>(a, s, pdl, smem_min, grouped);
-        case 8: return launch_d<8>(a, s, pdl, smem_min, grouped);
+        case 1: return launch_d<1>(a, s, pdl, grouped);
+        case 2: return launch_d<2>(a, s, pdl, grouped);
+        case 3: return launch_d<3>(a, s, pdl, grouped);
+        case 4: return launch_d<4>(a, s, pdl, grouped);
+        case 5: return launch_d<5>(a, s, pdl, grouped);
+        case 6: return launch_d<6>(a, s, pdl, grouped);
+        case 7: return launch_d<7>(a, s, pdl, grouped);
+        case 8: return launch_d<8>(a, s, pdl, grouped);
         default: return cudaErrorInvalidValue;
     }
 }

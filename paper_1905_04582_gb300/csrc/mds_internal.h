@@ -250,9 +250,8 @@ cudaError_t launch_pair_pass_f32(const PairArgs &a, int d, cudaStream_t s, bool 
 // one CTA each.
 // grouped: one CTA per SM whose groups of four warps each run a chunk
 // (pair_chunk_groups(d) groups); otherwise one chunk per CTA.
+cudaError_t launch_pair_chunks_f32(const PairArgs &a, int d, cudaStream_t s, bool pdl = true, bool grouped = false);
 cudaError_t launch_pair_chunks_batch(const ChunkBatchArgs &b, int d, bool long_runs, cudaStream_t s);
-cudaError_t launch_pair_chunks_f32(const PairArgs &a, int d, cudaStream_t s, bool pdl = true, int smem_min = 0,
-                                   bool grouped = false);
 int pair_chunk_smem_bytes(int d);
 int pair_chunk_blocks_per_sm(int d, bool grouped = false);  // chunk slots resident per SM
 int pair_chunk_groups(int d);
