@@ -1300,30 +1300,35 @@ bool small_traj(mds_ctx *c) {
 }
 
 // Enqueue one trajectory: start kernel, n_steps fused pair passes with their
-// leapfrog updates, end kernel (Metropolis when metropolis != 0).
+// leapfrog updates, end kernel (Metropolis when metropolis != 0).  n_iter > 1
+// (small_traj only): that many HMC iterations.
 int enqueue_trajectory(mds_ctx *c, int n_steps, double eps, int momentum_src, int u_src, int metropolis,
-                       uint64_t seed, cudaStream_t s) {
+                       uint64_t seed, cudaStream_t s, int n_iter = 1) {
     TrajArgs t = make_traj_args(c, n_steps, eps, momentum_src, seed, 0);
+    if (n_steps > 0 && small_traj(c)) {
+        SmallTrajArgs a{};
+        a.pair = pair_args(c);
+        a.pair.xcol2 = c->xcol2;
+        a.reduce = reduce_args(c, kModeHalfKick, eps);
+        const double scale = -1.0 / (c->sigma * c->sigma);
+        const float h = static_cast<float>(scale);
+        a.reduce.part_scale_df = make_float2(h, static_cast<float>(scale - static_cast<double>(h)));
+        a.traj = t;
+        a.accept = make_accept_args(c, n_steps, metropolis, u_src, seed, 0, 0, c->acc_out, c->dh_out,
+                                    static_cast<int64_t>(c->out_cap));
+        a.n_steps = n_steps;
+        for (int done = 0; done < n_iter; done += a.n_iter) {
+            a.n_iter = std::min(n_iter - done, kStIters);
+            cudaError_t e = launch_small_traj(a, c->d, s);
+            if (e != cudaSuccess) return fail(c, MDS_ERR_CUDA, "trajectory: %s", cudaGetErrorString(e));
+        }
+        return MDS_OK;
+    }
     int grid = 0;
     cudaError_t e = launch_traj_start(t, &grid, s);
     if (e != cudaSuccess) return fail(c, MDS_ERR_CUDA, "trajectory start: %s", cudaGetErrorString(e));
     c->start_grid = grid;
-    int k0 = 0;
-    if (n_steps > 1 && small_traj(c)) {
-        // all steps but the last (which gives the end's energies) in one launch
-        k0 = n_steps - 1;
-        SmallTrajArgs st{};
-        st.pair = pair_args(c);
-        st.pair.xcol2 = c->xcol2;
-        st.reduce = reduce_args(c, kModeKickDrift, eps);
-        const double scale = -1.0 / (c->sigma * c->sigma);
-        const float h = static_cast<float>(scale);
-        st.reduce.part_scale_df = make_float2(h, static_cast<float>(scale - static_cast<double>(h)));
-        st.n_steps = k0;
-        e = launch_small_traj(st, c->d, s);
-        if (e != cudaSuccess) return fail(c, MDS_ERR_CUDA, "trajectory steps: %s", cudaGetErrorString(e));
-    }
-    for (int k = k0; k < n_steps; ++k)
+    for (int k = 0; k < n_steps; ++k)
         CHECK(enqueue_pass(c, k + 1 < n_steps ? kModeKickDrift : kModeHalfKick, eps, s));
     AcceptArgs a = make_accept_args(c, n_steps, metropolis, u_src, seed, 0, grid, c->acc_out, c->dh_out,
                                     static_cast<int64_t>(c->out_cap));
@@ -1393,6 +1398,12 @@ int hmc_enqueue(mds_ctx *c, int n_iter, int n_steps, double eps, uint64_t seed, 
             CHECK(enqueue_trajectory(c, n_steps, eps, inj ? 2 : 1, inj ? 2 : 1, 1, seed, c->stream));
             c->hmc_pending++;
         }
+        return MDS_OK;
+    }
+    if (n_steps > 0 && small_traj(c)) {
+        // few launches without a graph: the iterations of a launch follow one another on the device
+        CHECK(enqueue_trajectory(c, n_steps, eps, inj ? 2 : 1, inj ? 2 : 1, 1, seed, c->stream, n_iter));
+        c->hmc_pending += n_iter;
         return MDS_OK;
     }
     // one HMC iteration as a CUDA graph, captured once per configuration

@@ -119,9 +119,11 @@ __device__ __forceinline__ bool block_far2(const float *box, const float2 (&c)[2
 
 // One tile for this lane (8 rows x 4 columns, column pairs in turn; see
 // pair_math.cuh tile_f32).  Returns the column pairs that took the far body.
-template <int D, bool MASKED, bool HELDOUT>
+// NQ < 4: a unit of fewer rows (16 NQ, the pointers and row_rel set to its
+// first).
+template <int D, bool MASKED, bool HELDOUT, int NQ = 4>
 __device__ __forceinline__ int tile_chunk(const PairArgs &a, const float4 *ys, const float2 *xjs, const float4 *xis,
-                                          int lane, int row_rel, int col_lo, int64_t ncol_valid, float2 (&racc)[4][D],
+                                          int lane, int row_rel, int col_lo, int64_t ncol_valid, float2 (&racc)[NQ][D],
                                           float *colp, float2 &e2, float2 &md, float2 &prod, const float *box) {
     constexpr int V = 2 * D;
     constexpr int P = Pow2<V>::value;
@@ -149,7 +151,7 @@ __device__ __forceinline__ int tile_chunk(const PairArgs &a, const float4 *ys, c
         if (far) {
             ++n_far;
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
+            for (int q = 0; q < NQ; ++q) {
                 const float4 yv = ys[(2 * q + cp) * 32 + (lane ^ (cp << 2))];
                 float4 xi[D];
 #pragma unroll
@@ -159,7 +161,7 @@ __device__ __forceinline__ int tile_chunk(const PairArgs &a, const float4 *ys, c
             }
         } else {
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
+            for (int q = 0; q < NQ; ++q) {
                 const float4 yv = ys[(2 * q + cp) * 32 + (lane ^ (cp << 2))];
                 float4 xi[D];
 #pragma unroll
@@ -212,10 +214,11 @@ __device__ __forceinline__ int tile_chunk(const PairArgs &a, const float4 *ys, c
 // the warp's Y quarter for even / odd q (tile layout, mds_internal.h), plus
 // (q / 2) * 64.  Returns the 64 x 8 blocks of the warp that took the far body
 // (0 or 2).
-template <int D, bool MASKED, bool HELDOUT>
+// NQ < 8: a unit of fewer rows (8 NQ), as in tile_chunk.
+template <int D, bool MASKED, bool HELDOUT, int NQ = 8>
 __device__ __forceinline__ int tile_tall(const PairArgs &a, const float4 *ys, const float2 *xjs, const float4 *xis,
                                          int lane, int ybe, int ybo, int row_rel, int col_lo, int64_t ncol_valid,
-                                         float2 (&racc)[8][D], float *colp, float2 &e2, float2 &md, float2 &prod,
+                                         float2 (&racc)[NQ][D], float *colp, float2 &e2, float2 &md, float2 &prod,
                                          const float *box) {
     constexpr int V = 2 * D;
     constexpr int P = Pow2<V>::value;
@@ -235,7 +238,7 @@ __device__ __forceinline__ int tile_tall(const PairArgs &a, const float4 *ys, co
     if constexpr (!MASKED) far = block_far2<D>(box, cj, a.far_d2);
     if (far) {
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
+        for (int q = 0; q < NQ; ++q) {
             const float4 yv = ys[(q >> 1) * 64 + ((q & 1) ? ybo : ybe)];
             float4 xi[D];
 #pragma unroll
@@ -250,7 +253,7 @@ __device__ __forceinline__ int tile_tall(const PairArgs &a, const float4 *ys, co
         }
     } else {
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
+        for (int q = 0; q < NQ; ++q) {
             const float4 yv = ys[(q >> 1) * 64 + ((q & 1) ? ybo : ybe)];
             float4 xi[D];
 #pragma unroll
@@ -297,12 +300,12 @@ __device__ __forceinline__ int tile_tall(const PairArgs &a, const float4 *ys, co
 
 // Row sums of one segment in the tall mapping into the warp's partial slot:
 // sums over the 8 column lanes of each row (3-level lane transpose).
-template <int D>
-__device__ __forceinline__ void flush_rows_tall(float2 (&racc)[8][D], int lane, float *rp) {
-    constexpr int VR = 16 * D;
+template <int D, int NQ = 8>
+__device__ __forceinline__ void flush_rows_tall(float2 (&racc)[NQ][D], int lane, float *rp) {
+    constexpr int VR = 2 * NQ * D;
     float rv[VR];
 #pragma unroll
-    for (int q = 0; q < 8; ++q)
+    for (int q = 0; q < NQ; ++q)
 #pragma unroll
         for (int k = 0; k < D; ++k) {
             rv[(q * D + k) * 2 + 0] = racc[q][k].x;
@@ -324,12 +327,12 @@ __device__ __forceinline__ void flush_rows_tall(float2 (&racc)[8][D], int lane, 
 // A warp's row sums of one segment (its 16 columns of every tile) into its
 // partial slot rp[64 * D]: sums over the 4 column lanes of each row
 // (lane transpose), then one store per value.
-template <int D>
-__device__ __forceinline__ void flush_rows(float2 (&racc)[4][D], int lane, float *rp) {
-    constexpr int VR = 8 * D;
+template <int D, int NQ = 4>
+__device__ __forceinline__ void flush_rows(float2 (&racc)[NQ][D], int lane, float *rp) {
+    constexpr int VR = 2 * NQ * D;
     float rv[VR];
 #pragma unroll
-    for (int q = 0; q < 4; ++q)
+    for (int q = 0; q < NQ; ++q)
 #pragma unroll
         for (int k = 0; k < D; ++k) {
             rv[(q * D + k) * 2 + 0] = racc[q][k].x;

@@ -351,15 +351,6 @@ struct ReduceArgs {
     unsigned *err;
 };
 
-// Kick-drift steps of a small problem in one launch (small_traj.cu).
-constexpr int kStMaxBlocks = 7;            // row blocks at most
-constexpr int kStMaxSmem = 224 * 1024;     // shared memory of a CTA at most
-struct SmallTrajArgs {
-    PairArgs pair;
-    ReduceArgs reduce;        // mode kModeKickDrift, part_scale_df -1/sigma^2
-    int32_t n_steps;
-};
-
 // The reduction runs kReduceQuarters CTAs per column block (16 items each)
 // plus one CTA for the scalars.
 constexpr int kReduceQuarters = 4;
@@ -423,6 +414,22 @@ struct AcceptArgs {
     unsigned *err;
 };
 cudaError_t launch_traj_end(const AcceptArgs &a, cudaStream_t s);
+
+// HMC iterations (or one trajectory) of a small problem in one launch (small_traj.cu).
+constexpr int kStMaxBlocks = 7;            // row blocks at most
+constexpr int kStMaxSmem = 220 * 1024;     // dynamic shared memory of a CTA at most
+constexpr int kStIters = 16;               // iterations of a launch at most (a few milliseconds)
+struct SmallTrajArgs {
+    PairArgs pair;
+    ReduceArgs reduce;        // part_scale_df -1/sigma^2
+    TrajArgs traj;
+    AcceptArgs accept;
+    int32_t n_steps;          // of each trajectory, at least 1
+    int32_t n_iter;
+};
+bool small_traj_fits(int64_t nt, int d);
+cudaError_t launch_small_traj(const SmallTrajArgs &a, int d, cudaStream_t s);
+
 // z (standard normal) and u (uniform) of sigma updates iter0 .. iter0 + n - 1.
 cudaError_t launch_sigma_draws(uint64_t seed, uint32_t chain, int64_t iter0, int n, double *z, double *u,
                                cudaStream_t s);
@@ -580,8 +587,6 @@ cudaError_t launch_ingest(const IngestArgs &a, cudaStream_t s);
 
 // Locations in: src (N x D, f32/f64) -> the state x (zero padded to n_pad)
 // and, on the FP32C path, the split layouts (quantum from *split).
-bool small_traj_fits(int64_t nt, int d);
-cudaError_t launch_small_traj(const SmallTrajArgs &a, int d, cudaStream_t s);
 cudaError_t launch_set_x(const void *src, bool src_f64, int64_t n, int64_t n_pad, int d, bool fp64, const XState &xs,
                          unsigned *err, HostPub *pub, cudaStream_t s);
 // Error word and scalars into pinned memory, the gradient (pairs: float2 (hi, lo), else double) into dst.
