@@ -97,7 +97,7 @@ struct mds_ctx {
                                   // bits come back with the next HMC read-back)
     uint64_t gen = 1;         // bumps whenever captured kernel arguments would change
     int start_grid = 0;
-    int small_fits = -1;      // small_traj_fits (device and size do not change), -1: not asked yet
+    int small_fits = -1;      // SmallUse bits that fit (device and size do not change), -1: not asked yet
 
     // device buffers
     float *y = nullptr;
@@ -1128,17 +1128,57 @@ int autotune(mds_ctx *c) {
     return MDS_OK;
 }
 
+// Whether trajectories (kSmallTraj), also evaluations (kSmallEval), run in one
+// launch: small FP32C problems whose target is the likelihood with the
+// isotropic prior, unless a shape of the pass is forced, a fault is injected
+// or the passes are timed one by one.
+enum SmallUse : int { kSmallTraj = 1, kSmallEval = 2 };
+bool small_use(mds_ctx *c, int what) {
+    if (c->fp64 || c->tree_on || sharded(c) || c->profiling || c->stamping || c->strip_req > 0 || c->chunk_req != 0)
+        return false;
+    if (c->small_fits < 0)
+        c->small_fits = (small_traj_fits(c->nt, c->d) ? kSmallTraj : 0) | (small_eval_fits(c->nt, c->d) ? kSmallEval : 0);
+    return (c->small_fits & what) && !getenv("MDS_STRIP") && !getenv("MDS_CHUNKS") && !getenv("MDS_FAULT");
+}
+
+// The arguments that both have in common.
+template <typename A>
+void small_args(const mds_ctx *c, int mode, double eps, A *a) {
+    a->pair = pair_args(c);
+    a->pair.xcol2 = c->xcol2;
+    a->reduce = reduce_args(c, mode, eps);
+    const double scale = -1.0 / (c->sigma * c->sigma);
+    const float h = static_cast<float>(scale);
+    a->reduce.part_scale_df = make_float2(h, static_cast<float>(scale - static_cast<double>(h)));
+}
+
+int small_eval(mds_ctx *c, HostPub *pub, void *dst, bool dst_f64) {
+    SmallEvalArgs a{};
+    small_args(c, kModeEval, 0.0, &a);
+    a.pub = pub;
+    a.dst = dst;
+    a.dst_f64 = dst_f64;
+    cudaError_t e = launch_small_eval(a, c->d, c->stream);
+    if (e != cudaSuccess) return fail(c, MDS_ERR_CUDA, "evaluation: %s", cudaGetErrorString(e));
+    return MDS_OK;
+}
+
 // Evaluate at the current x (gradient + scalars) and wait; the scalars are
-// then in c->pub, and the gradient in dst (device memory, if given).
-int evaluate(mds_ctx *c, void *dst = nullptr, bool dst_f64 = false) {
+// then in c->pub, and the gradient in dst (device memory, if given).  counted:
+// by the pass, which counts the far blocks.
+int evaluate(mds_ctx *c, void *dst = nullptr, bool dst_f64 = false, bool counted = false) {
     CHECK(ready(c));
     CHECK(autotune(c));
     if (fault_is("timeout")) {
         cudaError_t e = launch_wait_probe(c->err, c->stream);
         if (e != cudaSuccess) return fail(c, MDS_ERR_CUDA, "wait probe: %s", cudaGetErrorString(e));
     }
-    CHECK(enqueue_pass(c, kModeEval, 0.0, c->stream, fault_is("nan")));
-    CHECK(publish(c, dst, dst_f64));
+    if (!counted && small_use(c, kSmallEval)) {
+        CHECK(small_eval(c, c->pub, dst, dst_f64));
+    } else {
+        CHECK(enqueue_pass(c, kModeEval, 0.0, c->stream, fault_is("nan")));
+        CHECK(publish(c, dst, dst_f64));
+    }
     CU(cudaStreamSynchronize(c->stream));
     CHECK(published_status(c, "evaluation"));
     if (c->profiling) CHECK(harvest_prof(c));
@@ -1154,7 +1194,10 @@ int queue_start_eval(mds_ctx *c) {
     CHECK(autotune(c));
     if (c->grad_valid) return MDS_OK;
     if (c->profiling || std::getenv("MDS_FAULT")) return evaluate(c);
-    CHECK(enqueue_pass(c, kModeEval, 0.0, c->stream));
+    if (small_use(c, kSmallEval))
+        CHECK(small_eval(c, nullptr, nullptr, false));
+    else
+        CHECK(enqueue_pass(c, kModeEval, 0.0, c->stream));
     CU(cudaGetLastError());
     c->grad_valid = true;
     c->eval_unchecked = true;
@@ -1288,31 +1331,15 @@ AcceptArgs make_accept_args(const mds_ctx *c, int n_steps, int metropolis, int u
     return a;
 }
 
-// Whether trajectories run their steps in one launch: small FP32C problems
-// whose target is the likelihood with the isotropic prior, unless a shape of
-// the pass is forced or its passes are timed one by one.
-bool small_traj(mds_ctx *c) {
-    if (c->fp64 || c->tree_on || sharded(c) || c->profiling || c->stamping || c->strip_req > 0 || c->chunk_req != 0 ||
-        getenv("MDS_STRIP") || getenv("MDS_CHUNKS"))
-        return false;
-    if (c->small_fits < 0) c->small_fits = small_traj_fits(c->nt, c->d) ? 1 : 0;
-    return c->small_fits == 1;
-}
-
 // Enqueue one trajectory: start kernel, n_steps fused pair passes with their
 // leapfrog updates, end kernel (Metropolis when metropolis != 0).  n_iter > 1
-// (small_traj only): that many HMC iterations.
+// (small_use only): that many HMC iterations.
 int enqueue_trajectory(mds_ctx *c, int n_steps, double eps, int momentum_src, int u_src, int metropolis,
                        uint64_t seed, cudaStream_t s, int n_iter = 1) {
     TrajArgs t = make_traj_args(c, n_steps, eps, momentum_src, seed, 0);
-    if (n_steps > 0 && small_traj(c)) {
+    if (n_steps > 0 && small_use(c, kSmallTraj)) {
         SmallTrajArgs a{};
-        a.pair = pair_args(c);
-        a.pair.xcol2 = c->xcol2;
-        a.reduce = reduce_args(c, kModeHalfKick, eps);
-        const double scale = -1.0 / (c->sigma * c->sigma);
-        const float h = static_cast<float>(scale);
-        a.reduce.part_scale_df = make_float2(h, static_cast<float>(scale - static_cast<double>(h)));
+        small_args(c, kModeHalfKick, eps, &a);
         a.traj = t;
         a.accept = make_accept_args(c, n_steps, metropolis, u_src, seed, 0, 0, c->acc_out, c->dh_out,
                                     static_cast<int64_t>(c->out_cap));
@@ -1400,7 +1427,7 @@ int hmc_enqueue(mds_ctx *c, int n_iter, int n_steps, double eps, uint64_t seed, 
         }
         return MDS_OK;
     }
-    if (n_steps > 0 && small_traj(c)) {
+    if (n_steps > 0 && small_use(c, kSmallTraj)) {
         // few launches without a graph: the iterations of a launch follow one another on the device
         CHECK(enqueue_trajectory(c, n_steps, eps, inj ? 2 : 1, inj ? 2 : 1, 1, seed, c->stream, n_iter));
         c->hmc_pending += n_iter;
@@ -2389,7 +2416,7 @@ int reorder_ctx(mds_ctx *c, bool order_strips) {
         // one counted pass at the autotuned strip length, then the strips in
         // order of their cost
         if (order_strips && c->have_sigma) {
-            CHECK(evaluate(c));
+            CHECK(evaluate(c, nullptr, false, true));
             CHECK(order_strips_by_cost(c));
         }
     }
@@ -2407,7 +2434,7 @@ int mds_far_blocks(mds_ctx *c, int64_t *far, int64_t *total) {
         return fail(c, MDS_ERR_STATE, "queued HMC iterations: collect them first (mds_hmc_collect)");
     CHECK(ready(c));
     CHECK(autotune(c));  // so that the counted pass is the only one
-    CHECK(evaluate(c));
+    CHECK(evaluate(c, nullptr, false, true));
     int64_t v = 0;
     if (!c->fp64) {
         std::vector<int32_t> parts(static_cast<size_t>(c->n_strips) * kPairWarps);

@@ -117,11 +117,17 @@ __device__ __forceinline__ bool block_far2(const float *box, const float2 (&c)[2
     return __all_sync(0xffffffffu, fminf(g0, g1) >= far_d2);
 }
 
+// Place of value v (column v / D, coordinate v % D) where columns lie S floats apart.
+template <int D, int S>
+__device__ __forceinline__ int sum_at(int v) {
+    return S == D ? v : v / D * S + v % D;
+}
+
 // One tile for this lane (8 rows x 4 columns, column pairs in turn; see
 // pair_math.cuh tile_f32).  Returns the column pairs that took the far body.
 // NQ < 4: a unit of fewer rows (16 NQ, the pointers and row_rel set to its
-// first).
-template <int D, bool MASKED, bool HELDOUT, int NQ = 4>
+// first); S: floats between the column sums of neighbouring columns.
+template <int D, bool MASKED, bool HELDOUT, int NQ = 4, int S = D>
 __device__ __forceinline__ int tile_chunk(const PairArgs &a, const float4 *ys, const float2 *xjs, const float4 *xis,
                                           int lane, int row_rel, int col_lo, int64_t ncol_valid, float2 (&racc)[NQ][D],
                                           float *colp, float2 &e2, float2 &md, float2 &prod, const float *box) {
@@ -201,7 +207,7 @@ __device__ __forceinline__ int tile_chunk(const PairArgs &a, const float4 *ys, c
         if (writer) {
 #pragma unroll
             for (int i = 0; i < kHeld; ++i)
-                if (base + i < V) colp[(4 * lb + 2 * cp) * D + base + i] = colv[i];
+                if (base + i < V) colp[(4 * lb + 2 * cp) * S + sum_at<D, S>(base + i)] = colv[i];
         }
     }
     return n_far;
@@ -215,7 +221,7 @@ __device__ __forceinline__ int tile_chunk(const PairArgs &a, const float4 *ys, c
 // (q / 2) * 64.  Returns the 64 x 8 blocks of the warp that took the far body
 // (0 or 2).
 // NQ < 8: a unit of fewer rows (8 NQ), as in tile_chunk.
-template <int D, bool MASKED, bool HELDOUT, int NQ = 8>
+template <int D, bool MASKED, bool HELDOUT, int NQ = 8, int S = D>
 __device__ __forceinline__ int tile_tall(const PairArgs &a, const float4 *ys, const float2 *xjs, const float4 *xis,
                                          int lane, int ybe, int ybo, int row_rel, int col_lo, int64_t ncol_valid,
                                          float2 (&racc)[NQ][D], float *colp, float2 &e2, float2 &md, float2 &prod,
@@ -293,14 +299,14 @@ __device__ __forceinline__ int tile_tall(const PairArgs &a, const float4 *ys, co
     if (writer) {
 #pragma unroll
         for (int i = 0; i < kHeld; ++i)
-            if (base + i < V) colp[2 * lb * D + base + i] = colv[i];
+            if (base + i < V) colp[2 * lb * S + sum_at<D, S>(base + i)] = colv[i];
     }
     return far ? 2 : 0;
 }
 
 // Row sums of one segment in the tall mapping into the warp's partial slot:
 // sums over the 8 column lanes of each row (3-level lane transpose).
-template <int D, int NQ = 8>
+template <int D, int NQ = 8, int S = D>
 __device__ __forceinline__ void flush_rows_tall(float2 (&racc)[NQ][D], int lane, float *rp) {
     constexpr int VR = 2 * NQ * D;
     float rv[VR];
@@ -320,14 +326,14 @@ __device__ __forceinline__ void flush_rows_tall(float2 (&racc)[NQ][D], int lane,
     for (int i = 0; i < VR / 8; ++i) {
         const int v = base + i;
         const int h = v & 1, k = (v >> 1) % D, q = (v >> 1) / D;
-        rp[(2 * (la + 4 * q) + h) * D + k] = rv[i];
+        rp[(2 * (la + 4 * q) + h) * S + k] = rv[i];
     }
 }
 
 // A warp's row sums of one segment (its 16 columns of every tile) into its
 // partial slot rp[64 * D]: sums over the 4 column lanes of each row
 // (lane transpose), then one store per value.
-template <int D, int NQ = 4>
+template <int D, int NQ = 4, int S = D>
 __device__ __forceinline__ void flush_rows(float2 (&racc)[NQ][D], int lane, float *rp) {
     constexpr int VR = 2 * NQ * D;
     float rv[VR];
@@ -347,7 +353,7 @@ __device__ __forceinline__ void flush_rows(float2 (&racc)[NQ][D], int lane, floa
     for (int i = 0; i < VR / 4; ++i) {
         const int v = base + i;
         const int h = v & 1, k = (v >> 1) % D, q = (v >> 1) / D;
-        rp[(2 * (la + 8 * q) + h) * D + k] = rv[i];
+        rp[(2 * (la + 8 * q) + h) * S + k] = rv[i];
     }
 }
 

@@ -416,7 +416,7 @@ struct AcceptArgs {
 cudaError_t launch_traj_end(const AcceptArgs &a, cudaStream_t s);
 
 // HMC iterations (or one trajectory) of a small problem in one launch (small_traj.cu).
-constexpr int kStMaxBlocks = 7;            // row blocks at most
+constexpr int kStMaxBlocks = 8;            // row blocks at most
 constexpr int kStMaxSmem = 220 * 1024;     // dynamic shared memory of a CTA at most
 constexpr int kStIters = 16;               // iterations of a launch at most (a few milliseconds)
 struct SmallTrajArgs {
@@ -427,7 +427,17 @@ struct SmallTrajArgs {
     int32_t n_steps;          // of each trajectory, at least 1
     int32_t n_iter;
 };
+// One evaluation of a small problem.
+struct SmallEvalArgs {
+    PairArgs pair;
+    ReduceArgs reduce;        // part_scale_df -1/sigma^2
+    HostPub *pub;             // error bits and scalars for the host, or null
+    void *dst;                // the gradient for the caller (device), or null
+    bool dst_f64;
+};
 bool small_traj_fits(int64_t nt, int d);
+bool small_eval_fits(int64_t nt, int d);
+cudaError_t launch_small_eval(const SmallEvalArgs &a, int d, cudaStream_t s);
 cudaError_t launch_small_traj(const SmallTrajArgs &a, int d, cudaStream_t s);
 
 // z (standard normal) and u (uniform) of sigma updates iter0 .. iter0 + n - 1.

@@ -1,8 +1,8 @@
-"""Trajectories of small problems, whose steps run in one launch: the edges of
-its tiles, its units and its items per CTA, every dimension, a locality order,
-a fold and the isotropic prior, against the oracle's leapfrog with the
-tolerances of test_hmc_gpu; the same trajectory with a forced shape of the
-pass (a launch per pass and reduction) agrees to the same tolerance."""
+"""Evaluations and trajectories of small problems, each in one launch: the
+edges of its tiles, its units and its items per CTA, every dimension, a
+locality order, a fold and the isotropic prior, against the oracle with the
+tolerances of test_parity_gpu and test_hmc_gpu; the same with a forced shape
+of the pass (a launch per pass and reduction) agrees to the same tolerance."""
 import math
 
 import numpy as np
@@ -10,6 +10,7 @@ import pytest
 
 import oracle
 from paper_1905_04582_gb300 import workloads as W
+from gpu_util import TOL, grad_check, scalar_check
 
 pytestmark = pytest.mark.gpu
 
@@ -85,3 +86,41 @@ def test_small_hmc_device_draws_match_single_steps():
     np.testing.assert_array_equal(np.asarray(acc), acc_r)
     assert np.all(np.abs(np.asarray(dh) - dh_r) <= 2e-6 * abs(ll0) + 1e-6)
     np.testing.assert_allclose(x, xr, rtol=0, atol=2e-5 * (1 + np.abs(xr).max()))
+
+
+@pytest.mark.parametrize("n,d,mixture", [(2, 1, None), (17, 2, None), (63, 2, None), (64, 3, None), (65, 4, None),
+                                         (128, 1, (6, 0.3)), (200, 2, None), (257, 2, (6, 0.3)), (321, 8, None),
+                                         (385, 5, (3, 0.3)), (449, 6, None), (513, 2, (6, 0.3)), (641, 7, None),
+                                         (832, 1, None)])
+def test_small_evaluation_matches_oracle(n, d, mixture):
+    torch = pytest.importorskip("torch")
+    wl = W.custom(n, d, sigma=0.3 if mixture else 0.5, seed=700 + n + d, mixture=mixture)
+    x64 = wl.x_eval.astype(np.float32).astype(np.float64)
+    iu, ju = np.triu_indices(n, 1)
+    rng = np.random.default_rng(n)
+    pick = rng.choice(len(iu), size=max(1, len(iu) // 20), replace=False)
+    folds = [None] if n < 17 else [None, [(int(iu[q]), int(ju[q])) for q in pick]]
+    for reorder in (False, True):
+        for fold in folds:
+            keep = None if fold is None else oracle.keep_mask(n, fold)
+            ll_ref, _ = oracle.loglik(wl.y_packed, x64, wl.sigma, keep=keep)
+            ds_ref = oracle.dsigma(wl.y_packed, x64, wl.sigma, keep=keep)
+            g_ref, s_abs, s_sq = oracle.gradient(wl.y_packed, x64, wl.sigma, keep=keep, with_abs=True, with_sq=True)
+            m_pairs = n * (n - 1) // 2 if keep is None else int(keep.sum())
+            tol = TOL["fp32c"]
+            with model(wl) as m:
+                if reorder:
+                    m.reorder()
+                if fold is not None:
+                    m.set_heldout(fold)
+                out = torch.empty(n, d, device="cuda")
+                for how in ("host", "device f32", "device f64"):
+                    if how == "host":
+                        ll, g, ds = m.gradient()
+                    else:
+                        buf = out if how == "device f32" else out.double()
+                        ll, _, ds = m.gradient(out=buf)
+                        g = buf.double().cpu().numpy()
+                    scalar_check(ll, ll_ref, tol["ll"], scale=max(abs(ll_ref), m_pairs), what=f"L {how}")
+                    scalar_check(ds, ds_ref, tol["g"], scale=abs(ds_ref) + 2 * m_pairs / wl.sigma, what=f"ds {how}")
+                    grad_check(g, g_ref, s_abs, tol["g"], s_sq=s_sq, u=tol["u"], what=f"gradient {how}")
