@@ -4,6 +4,7 @@
 
 #include <cmath>
 #include <cstdint>
+#include <cstring>
 #include <cuda_runtime.h>
 
 namespace mds {
@@ -657,15 +658,21 @@ __host__ __device__ inline int split_bits(int d) { return d <= 1 ? 12 : d <= 4 ?
 // device (growth during a trajectory), so both pick the same quantum for the
 // same m.  False when q would leave [2^-100, 2^103] (x beyond FP32C range).
 __host__ __device__ inline bool choose_split(float m, int d, Split &sp) {
-    const double lim = static_cast<double>((1 << (split_bits(d) - 1)) - 1);
-    const double v = (static_cast<double>(m) > 1e-30 ? static_cast<double>(m) : 1e-30) * 4.0 / lim;
-    int e = 0;
-    const double f = frexp(v, &e);          // v = f 2^e, f in [0.5, 1)
-    const int ex = f == 0.5 ? e - 1 : e;    // ceil(log2 v)
+    const int lim = (1 << (split_bits(d) - 1)) - 1;
+    // ceil(log2(4 m / lim)) from the exponents and one comparison of the
+    // significands (exact): an FP64 division and frexp took 1.5 us of the
+    // locations' kernel, whatever its size
+    const float v = m > 1e-30f ? m : 1e-30f;
+    const float l = static_cast<float>(lim);
+    uint32_t bv, bl;
+    memcpy(&bv, &v, sizeof(bv));
+    memcpy(&bl, &l, sizeof(bl));
+    int ex = static_cast<int>(bv >> 23) - static_cast<int>(bl >> 23) + 2 + ((bv & 0x7fffffu) > (bl & 0x7fffffu) ? 1 : 0);
+    if (bv >= 0x7f800000u) ex = 0;  // infinite: the entries themselves are refused
     if (ex < -100 || ex > 103) return false;
     sp.q = ldexpf(1.0f, ex);
     sp.magic = ldexpf(1.5f, ex + 23);
-    sp.bound = static_cast<float>(lim * ldexp(1.0, ex));
+    sp.bound = ldexpf(l, ex);
     sp.resplit = 0;
     return true;
 }
