@@ -1880,8 +1880,10 @@ int mds_set_data(mds_ctx *c, const void *y, int dtype, int layout, int64_t ld, i
     } else {
         // host source: stage groups of row blocks through a device buffer
         // (a shard uploads only the rows of its tiles' row blocks)
-        const int64_t rows_per = kTile * std::max<int64_t>(1, (int64_t(64) << 20) / (kTile * n * eb));
-        const size_t stage_bytes = static_cast<size_t>(std::min<int64_t>(rows_per, n)) * n * eb;
+        // (rows come over with the source's stride: ld entries of a full matrix, at most n - 1 of a packed one)
+        const int64_t stride = a.packed ? n : ld;
+        const int64_t rows_per = kTile * std::max<int64_t>(1, (int64_t(64) << 20) / (kTile * stride * eb));
+        const size_t stage_bytes = static_cast<size_t>(std::min<int64_t>(rows_per, n)) * stride * eb;
         int64_t row_lo = 0, row_hi = n;
         if (c->shard_n > 1) {
             if (c->shard_t1 <= c->shard_t0) {
