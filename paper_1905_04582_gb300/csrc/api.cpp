@@ -142,7 +142,7 @@ struct mds_ctx {
     float *ho_y = nullptr;             // their y, set aside
     unsigned char *tile_ho = nullptr;  // [tiles] 1 where a tile holds a held-out pair
     double *lse_m = nullptr, *lse_s = nullptr;  // per pair running log-sum-exp of the densities
-    double *lpd_part = nullptr;        // kLpdParts partials + the result
+    double *lpd_part = nullptr;        // kLpdParts partials + the ticket of their sum
     int64_t lpd_draws = 0;
 
     // sigma updates (random walk on log sigma)
@@ -2175,7 +2175,10 @@ int mds_set_heldout(mds_ctx *c, const int64_t *pairs, int64_t n_pairs) {
         CHECK(dev_alloc_t(c, &c->tile_ho, static_cast<size_t>(c->tiles)));
         CU(cudaMemsetAsync(c->tile_ho, 0, static_cast<size_t>(c->tiles), c->stream));
     }
-    if (!c->lpd_part) CHECK(dev_alloc_t(c, &c->lpd_part, (kLpdParts + 1) * sizeof(double)));
+    if (!c->lpd_part) {
+        CHECK(dev_alloc_t(c, &c->lpd_part, (kLpdParts + 1) * sizeof(double)));
+        CU(cudaMemsetAsync(c->lpd_part + kLpdParts, 0, sizeof(double), c->stream));
+    }
     CHECK(dev_alloc_t(c, &c->ho_off, count * sizeof(int64_t)));
     CHECK(dev_alloc_t(c, &c->ho_pairs, count * sizeof(int2)));
     CHECK(dev_alloc_t(c, &c->ho_y, count * sizeof(float)));
@@ -2218,11 +2221,11 @@ int mds_lpd(mds_ctx *c, double *lpd, int64_t *draws) {
     CHECK(check_ctx(c));
     if (!lpd) return fail(c, MDS_ERR_INVALID_ARG, "lpd is NULL");
     if (c->lpd_draws == 0) return fail(c, MDS_ERR_STATE, "no draws accumulated (mds_lpd_accumulate)");
-    cudaError_t e = launch_lpd_sum(c->lse_m, c->lse_s, c->ho_count, static_cast<double>(c->lpd_draws),
-                                   c->lpd_part, c->lpd_part + kLpdParts, c->stream);
+    cudaError_t e = launch_lpd_sum(c->lse_m, c->lse_s, c->ho_count, static_cast<double>(c->lpd_draws), c->lpd_part,
+                                   reinterpret_cast<unsigned *>(c->lpd_part + kLpdParts), c->pub->scal, c->stream);
     if (e != cudaSuccess) return fail(c, MDS_ERR_CUDA, "lpd: %s", cudaGetErrorString(e));
-    CU(cudaMemcpyAsync(lpd, c->lpd_part + kLpdParts, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
     CU(cudaStreamSynchronize(c->stream));
+    *lpd = c->pub->scal[0];
     if (draws) *draws = c->lpd_draws;
     return MDS_OK;
 }

@@ -59,8 +59,11 @@ __global__ void __launch_bounds__(kLpdThreads, 2)
     double *tab = reinterpret_cast<double *>(lpd_smem);
     phi_table_load(tab);
     __syncthreads();
-    for (int64_t k = static_cast<int64_t>(blockIdx.x) * kLpdThreads + threadIdx.x; k < count;
-         k += static_cast<int64_t>(gridDim.x) * kLpdThreads) {
+    // a contiguous share per CTA: every SM then ends with the same number of
+    // warps (in a grid stride the last round filled some SMs and not others)
+    const int64_t per = (count + gridDim.x - 1) / gridDim.x;
+    const int64_t k1 = min(count, (blockIdx.x + 1) * per);
+    for (int64_t k = blockIdx.x * per + threadIdx.x; k < k1; k += kLpdThreads) {
         const int2 p = pairs[k];
         const float y = ho_y[k];
         const T *xi = x + static_cast<int64_t>(p.x) * d, *xj = x + static_cast<int64_t>(p.y) * d;
@@ -90,26 +93,32 @@ __global__ void __launch_bounds__(kLpdThreads, 2)
     }
 }
 
-// Block b sums the terms k = b, b + kLpdParts, ... in a fixed order (each
-// thread a strided subset, then a tree); the second launch (one block) sums
-// the kLpdParts partials the same way.
+// Block sum in a fixed order, in thread 0: shuffles, then the warps' sums.
 __device__ __forceinline__ double block_sum(double v, double *sm) {
-    sm[threadIdx.x] = v;
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = v;
     __syncthreads();
-    for (int o = kHoThreads / 2; o > 0; o >>= 1) {
-        if (static_cast<int>(threadIdx.x) < o) sm[threadIdx.x] += sm[threadIdx.x + o];
-        __syncthreads();
+    double t = sm[threadIdx.x % (kHoThreads / 32)];
+    if (threadIdx.x < 32) {
+#pragma unroll
+        for (int o = kHoThreads / 64; o >= 1; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
     }
-    return sm[0];
+    __syncthreads();
+    return t;
 }
 
-__global__ void lpd_partial_kernel(const double *lse_m, const double *lse_s, int64_t count, double log_draws,
-                                   double *part) {
-    __shared__ double sm[kHoThreads];
+// Block b sums the terms k = b kHoThreads + thread, in steps of the grid; the
+// last block to finish (a ticket that wraps to 0 for the next launch) sums the
+// kLpdParts partials, all in a fixed order, into out (pinned host memory).
+__global__ void __launch_bounds__(kHoThreads)
+    lpd_sum_kernel(const double *lse_m, const double *lse_s, int64_t count, double log_draws, double *part,
+                   unsigned *ticket, double *out) {
+    __shared__ double sm[kHoThreads / 32];
+    __shared__ bool last;
     double v = 0.0;
     for (int64_t k = static_cast<int64_t>(blockIdx.x) * kHoThreads + threadIdx.x; k < count;
-         k += static_cast<int64_t>(kLpdParts) * kHoThreads)
-    {
+         k += static_cast<int64_t>(kLpdParts) * kHoThreads) {
         // log 1 = 0 is left out: after the first draw every s is 1, and the FP64 log (about 40 instructions) would be
         // most of this kernel
         const double sc = lse_s[k];
@@ -117,15 +126,18 @@ __global__ void lpd_partial_kernel(const double *lse_m, const double *lse_s, int
         if (sc != 1.0) v += log(sc);
     }
     const double t = block_sum(v, sm);
-    if (threadIdx.x == 0) part[blockIdx.x] = t;
-}
-
-__global__ void lpd_final_kernel(const double *part, double *out) {
-    __shared__ double sm[kHoThreads];
-    double v = 0.0;
-    for (int k = threadIdx.x; k < kLpdParts; k += kHoThreads) v += part[k];
-    const double t = block_sum(v, sm);
-    if (threadIdx.x == 0) *out = t;
+    if (threadIdx.x == 0) {
+        part[blockIdx.x] = t;
+        __threadfence();
+        last = atomicInc(ticket, kLpdParts - 1) == kLpdParts - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    v = 0.0;
+    for (int k = threadIdx.x; k < kLpdParts; k += kHoThreads) v += __ldcg(part + k);
+    const double total = block_sum(v, sm);
+    if (threadIdx.x == 0) *out = total;
 }
 
 int grid_of(int64_t count) {
@@ -170,9 +182,8 @@ cudaError_t launch_lpd_accumulate(const void *x, bool fp64, int d, const int2 *p
 }
 
 cudaError_t launch_lpd_sum(const double *lse_m, const double *lse_s, int64_t count, double draws, double *part,
-                           double *out, cudaStream_t s) {
-    lpd_partial_kernel<<<kLpdParts, kHoThreads, 0, s>>>(lse_m, lse_s, count, log(draws), part);
-    lpd_final_kernel<<<1, kHoThreads, 0, s>>>(part, out);
+                           unsigned *ticket, double *out, cudaStream_t s) {
+    lpd_sum_kernel<<<kLpdParts, kHoThreads, 0, s>>>(lse_m, lse_s, count, std::log(draws), part, ticket, out);
     return cudaGetLastError();
 }
 

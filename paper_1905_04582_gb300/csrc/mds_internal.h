@@ -631,10 +631,11 @@ cudaError_t launch_lpd_accumulate(const void *x, bool fp64, int d, const int2 *p
                                   int64_t count, double sigma, bool first, double *lse_m, double *lse_s,
                                   unsigned *err, cudaStream_t s);
 // lpd-hat = sum over pairs of lse_m + log(lse_s) - log(draws) into *out
-// (fixed-order reduction; part holds kLpdParts doubles).
-constexpr int kLpdParts = 1024;
+// (fixed-order reduction; part holds kLpdParts doubles, ticket a zero that
+// stays zero between launches, out is pinned host memory).
+constexpr int kLpdParts = 304;
 cudaError_t launch_lpd_sum(const double *lse_m, const double *lse_s, int64_t count, double draws, double *part,
-                           double *out, cudaStream_t s);
+                           unsigned *ticket, double *out, cudaStream_t s);
 
 // Sharded evaluation (section 2.5: the pairwise sum split over workers, the
 // partial sums reduced).  pack: this shard's partials {L, dL/dsigma, sum r,
