@@ -5,11 +5,18 @@ that the FP64 pair arithmetic needs (pair_math64.cuh),
 phi and Phi the standard normal density and distribution function, on the
 nodes c = i / 64, i = 0 .. 608 (z up to 9.5): degree 5 in t = z - c, |t| <= 1/128,
 each the polynomial that interpolates the function at the 6 Chebyshev points
-of its interval (computed with 40 digits, coefficients rounded to FP64).
+of its interval (computed with 40 digits).  A node is 10 words of 64 bits, low
+half first:
+  F's coefficients of t^3, t^2, t, 1 and G's of t^3, t^2, t in FP64, G's
+  constant as an integer in units of 2^-52, {F's of t^5, F's of t^4} and
+  {G's of t^5, G's of t^4} in FP32 (t^4 <= 3.7e-9: their rounding is below
+  1e-16 of the value).
 
 Usage: python gen_phi_table.py > phi_table.h
 """
-from mpmath import cos, erfc, exp, log, mp, mpf, pi, sqrt
+import struct
+
+from mpmath import cos, erfc, exp, log, mp, mpf, nint, pi, sqrt
 
 mp.dps = 40
 PER_UNIT, NODES, DEG = 64, 609, 5
@@ -45,28 +52,38 @@ def fit(fn, c):
     return poly
 
 
+def f64(x):
+    return struct.unpack("<Q", struct.pack("<d", float(x)))[0]
+
+
+def f32(lo, hi):
+    return struct.unpack("<Q", struct.pack("<ff", float(lo), float(hi)))[0]
+
+
 def main():
     worst = [mpf(0), mpf(0)]
     rows = []
     for i in range(NODES):
         c = mpf(i) / PER_UNIT
-        row = []
+        co = []
         for q, fn in enumerate((f, g)):
             p = fit(fn, c)
             for u in (-1, mpf(-7) / 10, mpf(-1) / 4, mpf(1) / 3, mpf(8) / 10, 1):
                 t = u * HALF
                 v = sum(a * t ** k for k, a in enumerate(p))
                 worst[q] = max(worst[q], abs(v - fn(c + t)))
-            row += [float(a) for a in reversed(p)]
-        rows.append(row)
+            co.append(p)
+        a, b = co
+        rows.append([f64(a[3]), f64(a[2]), f64(a[1]), f64(a[0]), f64(b[3]), f64(b[2]), f64(b[1]),
+                     int(nint(b[0] * 2 ** 52)) & (2 ** 64 - 1), f32(a[5], a[4]), f32(b[5], b[4])])
     print("// Generated by gen_phi_table.py -- do not edit.")
-    print("// Node i, t = z - i/64: F = phi/Phi and G = log Phi as degree-5 polynomials, highest power first;")
+    print("// Node i, t = z - i/64: F = phi/Phi and G = log Phi as degree-5 polynomials (layout: see the generator);")
     print("// largest absolute error before the coefficients' rounding: F %.1e, G %.1e." % (worst[0], worst[1]))
     print("#pragma once")
-    print("constexpr int kPhiPerUnit = %d, kPhiNodes = %d, kPhiDeg = %d;" % (PER_UNIT, NODES, DEG))
-    print("__device__ const double g_phi_table[kPhiNodes * 2 * (kPhiDeg + 1)] = {")
+    print("constexpr int kPhiPerUnit = %d, kPhiNodes = %d, kPhiDeg = %d, kPhiRow = 10;" % (PER_UNIT, NODES, DEG))
+    print("__device__ const unsigned long long g_phi_table[kPhiNodes * kPhiRow] = {")
     for r in rows:
-        print(",".join("%.17g" % v for v in r) + ",")
+        print(",".join("0x%016xull" % v for v in r) + ",")
     print("};")
 
 

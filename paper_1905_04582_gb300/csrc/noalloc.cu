@@ -9,19 +9,23 @@
 // fixed file-scope array below, which every GPU that loads this library
 // holds until the process exits.
 //
-// Work split: one CTA per row i of the full N x N matrix Y (several rows in
-// turn beyond N = 8192); its threads stride over j != i, so every pair is
+// Work split: a CTA takes whole rows i of the full N x N matrix Y, in steps of
+// the grid; its threads stride over j != i, so every pair is
 // visited twice (once per end, as the per-row gradient sums of the paper's
 // Algorithm 2) and no column partials are needed.  The per-pair arithmetic is
 // that of the FP64 path (pair_math64.cuh), bound by the FP64 pipe; log Phi
 // and the other scalar terms are evaluated only for j > i.  A whole CTA per
 // row rather than a warp: the rows then come in pieces small enough to end
-// together on 152 SMs, and the table that each CTA reads is loaded while the
-// CTAs beside it compute.  Each block writes its partial sums of the scalar
+// together on 152 SMs.  The CTAs are resident all at once, two to four per SM,
+// and load the table once; how many, by what the last round leaves idle
+// (row_blocks): a CTA per row, left to the scheduler, took
+// 78 us at N = 600 (64), 400 at N = 2400 (351), D = 2, and 609 at N = 3001,
+// D = 3 (573, the shorter table included).  Each block writes its partial sums of the scalar
 // terms into the scratch array; a second, single-block kernel sums them in a
 // fixed order.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <cstdio>
@@ -47,6 +51,7 @@ static __device__ __align__(256) double g_noalloc_scratch[kNaMaxBlocks * kNaPart
 constexpr int kMaxDevices = 64;
 std::mutex g_na_mu;
 double *g_na_ptr[kMaxDevices] = {};
+int g_na_sms[kMaxDevices] = {};
 
 // Row sums: gradient in units of -sigma^2 (see pair_f64_kernel), then the scalars.
 template <int D>
@@ -58,6 +63,7 @@ struct RowSums {
 template <int D, bool SCALARS>
 __device__ __forceinline__ void row_part(const double *tab, const Sigma64 &sg, const double (&xi)[D],
                                          const double *x, const float *yrow, int64_t lo, int64_t hi, RowSums<D> &acc) {
+    int64_t log_units = 0;  // at most 512 terms of at most 0.7 * 2^52
     for (int64_t j0 = lo; j0 < hi; j0 += kNaThreads) {
         const bool in = j0 + threadIdx.x < hi;
         const int64_t j = in ? j0 + threadIdx.x : lo;
@@ -74,12 +80,13 @@ __device__ __forceinline__ void row_part(const double *tab, const Sigma64 &sg, c
         if constexpr (SCALARS) acc.v[D] = fma(w, w, acc.v[D]);
         const bool near = in && phi_near(sg, del);
         if (__any_sync(0xffffffffu, near)) {
-            double F, G;
-            phi_eval<SCALARS>(tab, sg, del, F, G);
-            F = near ? F : 0.0;
+            double F;
+            PhiLog G;
+            phi_eval<SCALARS>(tab, sg, del, near, F, G);
             if constexpr (SCALARS) {
                 acc.v[D + 1] = fma(F, del, acc.v[D + 1]);
-                acc.v[D + 2] += near ? G : 0.0;
+                acc.v[D + 2] = fma(G.slope, G.t, acc.v[D + 2]);
+                log_units += G.units;
             }
             w = fma(F, sg.neg_s, w);
         }
@@ -87,10 +94,11 @@ __device__ __forceinline__ void row_part(const double *tab, const Sigma64 &sg, c
 #pragma unroll
         for (int k = 0; k < D; ++k) acc.v[k] = fma(w, dl[k], acc.v[k]);
     }
+    if constexpr (SCALARS) acc.v[D + 2] = fma(static_cast<double>(log_units), kPhiUnit, acc.v[D + 2]);
 }
 
 template <int D>
-__global__ void __launch_bounds__(kNaThreads, 3) noalloc_rows_kernel(int64_t n, int rows, const float *y, int64_t ld,
+__global__ void __launch_bounds__(kNaThreads, 3) noalloc_rows_kernel(int64_t n, const float *y, int64_t ld,
                                                                      const double *x, Sigma64 sg, double *grad,
                                                                      double *part) {
     constexpr int V = D + 3, P = Pow2<V>::value;
@@ -101,8 +109,7 @@ __global__ void __launch_bounds__(kNaThreads, 3) noalloc_rows_kernel(int64_t n, 
     phi_table_load(tab);
     __syncthreads();
     double scalar = 0.0;  // threads D .. D + 2: the block's sums of the scalar terms
-    const int64_t i1 = min(n, static_cast<int64_t>(blockIdx.x + 1) * rows);
-    for (int64_t i = static_cast<int64_t>(blockIdx.x) * rows; i < i1; ++i) {
+    for (int64_t i = blockIdx.x; i < n; i += gridDim.x) {
         RowSums<D> acc;
 #pragma unroll
         for (int q = 0; q < P; ++q) acc.v[q] = 0.0;
@@ -147,9 +154,24 @@ __global__ void noalloc_sum_kernel(int nblocks, double *part) {
     if (threadIdx.x < 3) part[kNaMaxBlocks * kNaParts + threadIdx.x] = sm[threadIdx.x][0];
 }
 
+// CTAs for n rows: k per SM, k = 4, 3 or 2.  An SM's FP64 pipes are shared, so
+// its time is k times its largest CTA's number of rows, ceil(n / (k SMs)):
+// the k with the smallest product, more CTAs (latency) where they are equal.
+int64_t row_blocks(int64_t n, int sms) {
+    int64_t best = 0, cost = 0;
+    for (int64_t k = 4; k >= 2; --k) {
+        const int64_t c = k * ((n + k * sms - 1) / (k * sms));
+        if (best == 0 || c < cost) {
+            best = k;
+            cost = c;
+        }
+    }
+    return std::min<int64_t>(n, std::min<int64_t>(best * sms, kNaMaxBlocks));
+}
+
 // Device address of the scratch array on the current device (looked up once
 // per device; host code cannot use the symbol itself as a device pointer).
-int scratch_address(double **out) {
+int scratch_address(double **out, int *sms) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) {
@@ -168,9 +190,15 @@ int scratch_address(double **out) {
             mds::set_thread_error("mds_loglik_grad_noalloc: cudaGetSymbolAddress: %s", cudaGetErrorString(e));
             return MDS_ERR_CUDA;
         }
+        e = cudaDeviceGetAttribute(&g_na_sms[dev], cudaDevAttrMultiProcessorCount, dev);
+        if (e != cudaSuccess) {
+            mds::set_thread_error("mds_loglik_grad_noalloc: cudaDeviceGetAttribute: %s", cudaGetErrorString(e));
+            return MDS_ERR_CUDA;
+        }
         g_na_ptr[dev] = static_cast<double *>(p);
     }
     *out = g_na_ptr[dev];
+    *sms = g_na_sms[dev];
     return MDS_OK;
 }
 
@@ -192,11 +220,11 @@ extern "C" int mds_loglik_grad_noalloc(int64_t n, int32_t d, const float *y, int
                               static_cast<long long>(n), static_cast<long long>(kNaMaxN));
         return MDS_ERR_INVALID_ARG;
     }
-    const int rows = static_cast<int>((n + kNaMaxBlocks - 1) / kNaMaxBlocks);
-    const int64_t nblocks = (n + rows - 1) / rows;
     double *part = nullptr;
-    int st = scratch_address(&part);
+    int sms = 0;
+    int st = scratch_address(&part, &sms);
     if (st != MDS_OK) return st;
+    const int64_t nblocks = row_blocks(n, sms);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     cudaError_t e = cudaSuccess;
     const Sigma64 sg = sigma64(sigma);
@@ -206,7 +234,7 @@ extern "C" int mds_loglik_grad_noalloc(int64_t n, int32_t d, const float *y, int
         e = mds::raise_dyn_smem(reinterpret_cast<const void *>(noalloc_rows_kernel<DD>), kPhiBytes);              \
         if (e == cudaSuccess)                                                                                     \
             noalloc_rows_kernel<DD>                                                                               \
-                <<<static_cast<int>(nblocks), kNaThreads, kPhiBytes, s>>>(n, rows, y, ld, x, sg, grad, part);    \
+                <<<static_cast<int>(nblocks), kNaThreads, kPhiBytes, s>>>(n, y, ld, x, sg, grad, part);          \
         break;
         MDS_NA_CASE(1) MDS_NA_CASE(2) MDS_NA_CASE(3) MDS_NA_CASE(4)
         MDS_NA_CASE(5) MDS_NA_CASE(6) MDS_NA_CASE(7) MDS_NA_CASE(8)

@@ -6,13 +6,17 @@
 // every 64 cycles, so a pair costs its FP64 instructions and everything else
 // (integer, FP32, shared memory, MUFU) is nearly free beside them.  With
 // CUDA's sqrt, division, erfc, exp and log1p a pair took about 187 of them at
-// D = 2; the forms below take 19, and 14 more where Phi matters:
+// D = 2; the forms below take 19, and 11 more where Phi matters:
 //  - 1/delta and delta: one cubic (Halley) step from the hardware's
 //    reciprocal-root seed, then delta corrected by its own residual
 //    d^2 - s^2, which an FMA gives exactly: 8, for a root and a division;
 //  - phi/Phi and log Phi as functions of z alone, piecewise polynomials of
 //    degree 5 on nodes 1/64 apart (phi_table.h, absolute error 9e-18), the
-//    table in shared memory: 13, for an exp, an erfc, a division and a log1p.
+//    table in shared memory: 11, for an exp, an erfc, a division and a log1p.
+//    The two highest powers are FP32 (t^4 <= 3.7e-9 takes their rounding below
+//    1e-16 of F and G; errors against 40 digits: F 1.3e-17 rms as in FP64
+//    throughout), t and their sum carried over by moving bits; G's constant is
+//    summed as an integer, so that its last step is the sum's own FMA.
 //    What matters is their absolute error: beside phi/Phi the weight holds
 //    (delta - y)/sigma, whose rounding is at least 2^-53 z;
 //  - beyond z = 9.5 both are dropped: phi/Phi < 1.1e-20 there, five orders
@@ -22,8 +26,9 @@
 //  - y, an FP32 value, widened by moving bits (a conversion instruction would
 //    cost as much as an FMA).
 // Measured (GB300, whole calls, the errors against 64 bits unchanged): L,
-// dL/dX and dL/dsigma at N = 5392, D = 2, caller's order, 4.35 -> 1.02 ms; the
-// allocation-free call at N = 3001, D = 3, 2.84 -> 0.61 ms.
+// dL/dX and dL/dsigma at N = 5392, D = 2, caller's order, 4.35 -> 0.97 ms (1.00
+// with every power in FP64); the allocation-free call at N = 3001, D = 3,
+// 2.84 -> 0.57 ms.
 #pragma once
 
 #include <cstdint>
@@ -34,15 +39,15 @@ namespace {
 
 #include "phi_table.h"
 
-constexpr int kPhiRow = 2 * (kPhiDeg + 1);                  // doubles per node
-constexpr int kPhiBytes = kPhiNodes * kPhiRow * 8;          // 58,464
-static_assert(kPhiDeg == 5 && kPhiPerUnit == 64 && kPhiBytes % 16 == 0, "phi_eval is written for this table");
+constexpr int kPhiBytes = kPhiNodes * kPhiRow * 8;  // 48,720
+static_assert(kPhiDeg == 5 && kPhiPerUnit == 64 && kPhiRow == 10 && kPhiBytes % 16 == 0,
+              "phi_eval is written for this table");
 
 // The table into shared memory (16-byte aligned), by all threads of the CTA;
 // the caller synchronises.
 __device__ __forceinline__ void phi_table_load(double *tab) {
-    const double2 *src = reinterpret_cast<const double2 *>(g_phi_table);
-    double2 *dst = reinterpret_cast<double2 *>(tab);
+    const ulonglong2 *src = reinterpret_cast<const ulonglong2 *>(g_phi_table);
+    ulonglong2 *dst = reinterpret_cast<ulonglong2 *>(tab);
     for (int i = threadIdx.x; i < kPhiBytes / 16; i += blockDim.x) dst[i] = src[i];
 }
 
@@ -116,25 +121,58 @@ __device__ __forceinline__ uint32_t phi_node(const Sigma64 &sg, double del, doub
     return i;
 }
 
-__device__ __forceinline__ double phi_poly(const double2 *c, double t) {
-    const double2 c54 = c[0], c32 = c[1], c10 = c[2];
-    return fma(fma(fma(fma(fma(c54.x, t, c54.y), t, c32.x), t, c32.y), t, c10.x), t, c10.y);
+// t in FP32 (truncated; 0 below the FP32 range): the same bits, moved.
+__device__ __forceinline__ float narrow(double t) {
+    const uint32_t hi = static_cast<uint32_t>(__double2hiint(t)), lo = static_cast<uint32_t>(__double2loint(t));
+    const uint32_t m = hi & 0x7fffffffu;
+    const uint32_t b = (hi & 0x80000000u) | ((m - 0x38000000u) << 3) | (lo >> 29);
+    return m < 0x38100000u ? 0.f : __uint_as_float(b);
 }
 
-// F = phi(z)/Phi(z), G = log Phi(z) at z = del / sigma, phi_near(del); WANT_G false leaves G alone.
-template <bool WANT_G>
-__device__ __forceinline__ void phi_eval(const double *tab, const Sigma64 &sg, double del, double &F, double &G) {
+// G = log Phi(z) in two parts: slope * t + units * 2^-52.
+struct PhiLog {
+    double slope, t;
+    int64_t units;
+};
+constexpr double kPhiUnit = 0x1p-52;
+
+template <bool WANT_F, bool WANT_G>
+__device__ __forceinline__ void phi_parts(const double *tab, const Sigma64 &sg, double del, bool near, double &F,
+                                          PhiLog &G) {
     double t;
     const double2 *row = reinterpret_cast<const double2 *>(tab + phi_node(sg, del, t) * kPhiRow);
-    F = phi_poly(row, t);
-    if constexpr (WANT_G) G = phi_poly(row + 3, t);
+    t = near ? t : 0.0;
+    const float4 high = *reinterpret_cast<const float4 *>(row + 4);
+    const float tf = narrow(t);
+    if constexpr (WANT_F) {
+        const double2 f32 = row[0], f10 = row[1];
+        const double u = widen_signed(fmaf(high.x, tf, high.y));
+        F = fma(fma(fma(fma(u, t, f32.x), t, f32.y), t, f10.x), t, f10.y);
+        F = near ? F : 0.0;
+    }
+    if constexpr (WANT_G) {
+        const double2 g32 = row[2], g10 = row[3];
+        const double u = widen_signed(fmaf(high.z, tf, high.w));
+        G.slope = fma(fma(fma(u, t, g32.x), t, g32.y), t, g10.x);
+        G.t = t;
+        G.units = near ? __double_as_longlong(g10.y) : 0;
+    }
 }
 
-// log Phi(z) alone.
+// F = phi(z)/Phi(z) and G at z = del / sigma; 0 where near is false (near:
+// phi_near(del)); WANT_G false leaves G alone.
+template <bool WANT_G>
+__device__ __forceinline__ void phi_eval(const double *tab, const Sigma64 &sg, double del, bool near, double &F,
+                                         PhiLog &G) {
+    phi_parts<true, WANT_G>(tab, sg, del, near, F, G);
+}
+
+// log Phi(z) alone, phi_near(del).
 __device__ __forceinline__ double phi_log(const double *tab, const Sigma64 &sg, double del) {
-    double t;
-    const uint32_t i = phi_node(sg, del, t);
-    return phi_poly(reinterpret_cast<const double2 *>(tab + i * kPhiRow) + 3, t);
+    double F;
+    PhiLog G;
+    phi_parts<false, true>(tab, sg, del, true, F, G);
+    return fma(G.slope, G.t, static_cast<double>(G.units) * kPhiUnit);
 }
 
 }  // namespace
