@@ -56,7 +56,7 @@ def fp32_ops_per_pair(d, far_frac=0.0, chunked=True):
     return (1.0 - far_frac) * near + far_frac * far
 
 
-PAIR_KERNEL_SOURCES = ("pair_kernel.cu", "chunk_kernel.cu", "pair_math.cuh", "mills_ratio_coeffs.h")
+PAIR_KERNEL_SOURCES = ("pair_kernel.cu", "chunk_kernel.cu", "chunk_tile.cuh", "pair_math.cuh", "mills_ratio_coeffs.h")
 # the part of mds_internal.h the pair kernel is compiled from: the tile
 # geometry through the end of its argument struct, and the error bits
 PAIR_KERNEL_INTERNAL = (("// Tile geometry of the pair pass.", "cudaError_t launch_pair_batch"),)

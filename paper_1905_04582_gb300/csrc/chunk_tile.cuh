@@ -309,6 +309,7 @@ __device__ __forceinline__ int tile_tall(const PairArgs &a, const float4 *ys, co
 template <int D, int NQ = 8, int S = D>
 __device__ __forceinline__ void flush_rows_tall(float2 (&racc)[NQ][D], int lane, float *rp) {
     constexpr int VR = 2 * NQ * D;
+    static_assert(VR % 8 == 0, "three halvings of the values");
     float rv[VR];
 #pragma unroll
     for (int q = 0; q < NQ; ++q)
@@ -336,6 +337,7 @@ __device__ __forceinline__ void flush_rows_tall(float2 (&racc)[NQ][D], int lane,
 template <int D, int NQ = 4, int S = D>
 __device__ __forceinline__ void flush_rows(float2 (&racc)[NQ][D], int lane, float *rp) {
     constexpr int VR = 2 * NQ * D;
+    static_assert(VR % 4 == 0, "two halvings of the values");
     float rv[VR];
 #pragma unroll
     for (int q = 0; q < NQ; ++q)
