@@ -3171,7 +3171,7 @@ struct mds_batch {
     int64_t max_nd = 0;
     uint64_t gen = 1;
     cudaGraphExec_t graph = nullptr;
-    std::tuple<uint64_t, int> graph_key{};
+    std::tuple<uint64_t, int, std::vector<uint64_t>> graph_key{};
     // the chains' scalars, counters and error words, each chain's after the
     // other's, so that one copy or memset serves all of them
     double *scal_all = nullptr;
@@ -3623,6 +3623,7 @@ int mds_batch_set_data(mds_batch *b, int32_t dataset, const void *y, int dtype, 
     for (int c = 0; c < b->chains[dataset]; ++c) {
         mds_ctx *x = b->ctx[b->chain0[dataset] + c];
         x->have_data = c0->have_data;
+        if (x->y != c0->y) x->gen++;
         x->y = c0->y;  // the first chain may have repacked Y into a new buffer (its slot order)
         x->grad_valid = false;
     }
@@ -3725,12 +3726,13 @@ int mds_batch_hmc(mds_batch *b, int n_iter, int n_steps, const double *eps, uint
                           b->stream));
     BCU(cudaMemcpyAsync(b->tcfg, tc.data(), total * sizeof(TrajArgs), cudaMemcpyHostToDevice, b->stream));
     BCU(cudaMemcpyAsync(b->acfg, ac.data(), total * sizeof(AcceptArgs), cudaMemcpyHostToDevice, b->stream));
-    const auto key = std::make_tuple(b->gen, n_steps);
+    // chunked passes are captured with each chain's arguments by value (sigma's
+    // constants, the pointer to Y): a chain's gen counts their changes
+    std::vector<uint64_t> gens;
+    if (b->strip < 0)
+        for (const mds_ctx *c : b->ctx) gens.push_back(c->gen);
+    const auto key = std::make_tuple(b->gen, n_steps, gens);
     if (!b->graph || key != b->graph_key || max_grid != b->max_start_grid || max_nd != b->max_nd) {
-        if (b->graph) {
-            cudaGraphExecDestroy(b->graph);
-            b->graph = nullptr;
-        }
         cudaGraph_t g = nullptr;
         BCU(cudaStreamBeginCapture(b->cap_stream, cudaStreamCaptureModeThreadLocal));
         cudaError_t e = launch_traj_start_batch(b->tcfg, total, max_grid, b->d, b->cap_stream);
@@ -3747,9 +3749,22 @@ int mds_batch_hmc(mds_batch *b, int n_iter, int n_steps, const double *eps, uint
             return st;
         }
         if (e != cudaSuccess) return bfail(b, MDS_ERR_CUDA, "graph capture: %s", cudaGetErrorString(e));
-        e = cudaGraphInstantiate(&b->graph, g, 0);
+        if (b->graph) {
+            // same launches with new arguments (sigma, Y): update the
+            // instantiated graph in place; otherwise instantiate afresh
+            cudaGraphExecUpdateResultInfo info;
+            if (cudaGraphExecUpdate(b->graph, g, &info) != cudaSuccess) {
+                cudaGetLastError();
+                cudaGraphExecDestroy(b->graph);
+                b->graph = nullptr;
+            }
+        }
+        if (!b->graph) e = cudaGraphInstantiate(&b->graph, g, 0);
         cudaGraphDestroy(g);
-        if (e != cudaSuccess) return bfail(b, MDS_ERR_CUDA, "graph instantiate: %s", cudaGetErrorString(e));
+        if (e != cudaSuccess) {
+            b->graph = nullptr;
+            return bfail(b, MDS_ERR_CUDA, "graph instantiate: %s", cudaGetErrorString(e));
+        }
         b->graph_key = key;
         b->max_start_grid = max_grid;
         b->max_nd = max_nd;
