@@ -3239,15 +3239,19 @@ int bdev_alloc(mds_batch *b, P **p, size_t bytes) {
     return MDS_OK;
 }
 
-// A device table from its host copy, if it differs from what the device holds
-// (a copy from pageable memory has left the source when the call returns).
+// A device table from its host copy, if it differs from what the device holds.
+// The copy is done when the call returns, so that what `sent` says holds on
+// any stream that a later call uses.
 template <typename T>
 int batch_upload(mds_batch *b, int slot, T *dev, const std::vector<T> &v) {
     const size_t bytes = v.size() * sizeof(T);
     std::vector<unsigned char> &sent = b->sent[slot];
     if (sent.size() == bytes && (bytes == 0 || std::memcmp(sent.data(), v.data(), bytes) == 0)) return MDS_OK;
     sent.clear();
-    if (bytes) BCU(cudaMemcpyAsync(dev, v.data(), bytes, cudaMemcpyHostToDevice, b->stream));
+    if (bytes) {
+        BCU(cudaMemcpyAsync(dev, v.data(), bytes, cudaMemcpyHostToDevice, b->stream));
+        BCU(cudaStreamSynchronize(b->stream));
+    }
     const unsigned char *src = reinterpret_cast<const unsigned char *>(v.data());
     sent.assign(src, src + bytes);
     return MDS_OK;
@@ -3691,7 +3695,10 @@ int mds_batch_hmc(mds_batch *b, int n_iter, int n_steps, const double *eps, uint
         CHECK(batch_evaluate(b));
     else
         CHECK(batch_autotune(b));
-    if (n_iter == 0) return MDS_OK;
+    if (n_iter == 0) {
+        BCU(cudaStreamSynchronize(b->stream));
+        return MDS_OK;
+    }
     const int total = static_cast<int>(b->ctx.size());
     if (static_cast<size_t>(n_iter) > b->out_cap) {
         if (b->acc_out) cudaFree(b->acc_out);
