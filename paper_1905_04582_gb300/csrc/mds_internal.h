@@ -657,7 +657,8 @@ __host__ __device__ inline int split_bits(int d) { return d <= 1 ? 12 : d <= 4 ?
 // (2^(B-1) - 1) q >= 4 m (4x headroom for the moves of a trajectory).  The
 // same function runs on the host (locations set by the caller) and on the
 // device (growth during a trajectory), so both pick the same quantum for the
-// same m.  False when q would leave [2^-100, 2^103] (x beyond FP32C range).
+// same m.  False when q would leave [2^-100, 2^103] (x beyond the FP32C range, an
+// infinite m among them).
 __host__ __device__ inline bool choose_split(float m, int d, Split &sp) {
     const int lim = (1 << (split_bits(d) - 1)) - 1;
     // ceil(log2(4 m / lim)) from the exponents and one comparison of the
@@ -669,7 +670,6 @@ __host__ __device__ inline bool choose_split(float m, int d, Split &sp) {
     memcpy(&bv, &v, sizeof(bv));
     memcpy(&bl, &l, sizeof(bl));
     int ex = static_cast<int>(bv >> 23) - static_cast<int>(bl >> 23) + 2 + ((bv & 0x7fffffu) > (bl & 0x7fffffu) ? 1 : 0);
-    if (bv >= 0x7f800000u) ex = 0;  // infinite: the entries themselves are refused
     if (ex < -100 || ex > 103) return false;
     sp.q = ldexpf(1.0f, ex);
     sp.magic = ldexpf(1.5f, ex + 23);

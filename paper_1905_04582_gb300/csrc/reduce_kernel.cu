@@ -143,6 +143,17 @@ __device__ __forceinline__ void load_coords(const T *p, bool ok, T (&v)[D]) {
     }
 }
 
+// The running max |x| at a trajectory's end, for the growth of the quantum
+// (one thread).  An infinite one is of a diverged trajectory, which is reported
+// as non-finite: the quantum stays, as it holds for the locations that a
+// rejection restores, and the maximum goes back to that quantum's bound.
+__device__ __forceinline__ float grown_max(const XState &xs, const Split &sp) {
+    const float m = __uint_as_float(*xs.xmax_bits);
+    if (isfinite(m)) return m;
+    *xs.xmax_bits = __float_as_uint(sp.bound);
+    return sp.bound;
+}
+
 // ROWS items per CTA (kRedRows or a whole block), Jq counting CTAs.
 template <typename T, int D, int ROWS>
 __device__ __forceinline__ void reduce_body(const ReduceArgs &a, int mode, int Jq) {
@@ -194,7 +205,7 @@ __device__ __forceinline__ void reduce_body(const ReduceArgs &a, int mode, int J
         if constexpr (kF32) {
             if (tid == 0 && mode == kModeHalfKick) {
                 Split sp = *a.xs.split;
-                const float m = __uint_as_float(*a.xs.xmax_bits);
+                const float m = grown_max(a.xs, sp);
                 int rs = 0;
                 if (m > sp.bound) {
                     Split ns;
@@ -277,7 +288,7 @@ __device__ __forceinline__ void reduce_body(const ReduceArgs &a, int mode, int J
                     // grow the quantum if the running max |x| outgrew it; the
                     // trajectory-end kernel rewrites the layouts
                     Split sp = *a.xs.split;
-                    const float m = __uint_as_float(*a.xs.xmax_bits);
+                    const float m = grown_max(a.xs, sp);
                     int rs = 0;
                     if (m > sp.bound) {
                         Split ns;
@@ -1011,10 +1022,9 @@ __global__ void repack_kernel(const float *old_y, float *new_y, const int32_t *m
 
 // Locations from the caller.  FP32C: the split quantum follows from max |x|
 // of the incoming values; every CTA derives the same quantum by the
-// host/device rule (choose_split, one thread of it: the rule's FP64 division
-// by every warp took longer than the rest of the kernel) and CTA 0 stores it.
-// Outside the FP32C range nothing is written and the range bit is raised, so
-// the previous state stays intact.  The call's error bits go to `pub` (pinned
+// host/device rule (choose_split, one thread of it) and CTA 0 stores it.
+// Outside the FP32C range, finite FP64 values beyond FP32 included, nothing is
+// written and the range bit is raised, so the previous state stays intact.  The call's error bits go to `pub` (pinned
 // host memory: the host reads them after its wait, without a copy); bits that
 // earlier work left in the context's error word are cleared.
 //
@@ -1023,6 +1033,17 @@ __global__ void repack_kernel(const float *old_y, float *new_y, const int32_t *m
 // up to kSetXOne elements.  Beyond, xmax_kernel runs just before.
 constexpr int kSetXThreads = 512;
 constexpr int64_t kSetXOne = 32768;
+
+// |v| in FP32; a finite FP64 value beyond FP32 counts as FP32's largest (out
+// of the split's range), so that Inf means an infinite entry.
+template <typename S>
+__device__ __forceinline__ float abs_f32(S v) {
+    const float a = fabsf(static_cast<float>(v));
+    if constexpr (sizeof(S) == 8) {
+        if (isinf(a) && !isinf(v)) return FLT_MAX;
+    }
+    return a;
+}
 
 template <typename S>
 __device__ __forceinline__ float abs_max(const S *src, int64_t count) {
@@ -1036,11 +1057,11 @@ __device__ __forceinline__ float abs_max(const S *src, int64_t count) {
     for (int64_t e = threadIdx.x; e < vecs; e += kSetXThreads) {
         const Vec w = reinterpret_cast<const Vec *>(src)[e];
 #pragma unroll
-        for (int i = 0; i < kV; ++i) m = fmaxf(m, fabsf(static_cast<float>(w.v[i])));
+        for (int i = 0; i < kV; ++i) m = fmaxf(m, abs_f32(w.v[i]));
     }
 #pragma unroll 8
     for (int64_t e = vecs * kV + threadIdx.x; e < count; e += kSetXThreads)
-        m = fmaxf(m, fabsf(static_cast<float>(src[e])));
+        m = fmaxf(m, abs_f32(src[e]));
     return m;
 }
 
@@ -1059,8 +1080,9 @@ __global__ void __launch_bounds__(kSetXThreads)
         else
             m = __uint_as_float(*xs.xmax_bits);
         if (threadIdx.x == 0) {
+            // infinite entries are refused below, as NaN entries are (any quantum will do)
             Split s1{};
-            ok_s = choose_split(m, d, s1);
+            ok_s = choose_split(isinf(m) ? 1.f : m, d, s1);
             sp_s = s1;
         }
         __syncthreads();
@@ -1113,7 +1135,7 @@ __global__ void xmax_kernel(const T *x, int64_t count, unsigned *out) {
     float m = 0.f;
     for (int64_t e = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; e < count;
          e += static_cast<int64_t>(gridDim.x) * blockDim.x)
-        m = fmaxf(m, fabsf(static_cast<float>(x[e])));
+        m = fmaxf(m, abs_f32(x[e]));
     m = block_max<256>(m, sm);
     if (threadIdx.x == 0 && m > 0.f) atomicMax(out, __float_as_uint(m));
 }

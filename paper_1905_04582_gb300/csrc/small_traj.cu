@@ -516,7 +516,9 @@ __global__ void __launch_bounds__(32 * st_warps<D>(), 1) small_traj_kernel(const
                 x_s[e] = x0_s[e];
         }
         // the split quantum grows when the trajectory outgrew its bound (the same rule in every CTA)
-        const float m = static_cast<float>(sum_s[kPartXmax]);
+        // (but for an infinite maximum: a diverged trajectory, reported as non-finite)
+        float m = static_cast<float>(sum_s[kPartXmax]);
+        if (isinf(m)) m = xmax = sp.bound;
         if (m > sp.bound) {
             Split ns;
             if (choose_split(m, D, ns))
@@ -537,7 +539,8 @@ __global__ void __launch_bounds__(32 * st_warps<D>(), 1) small_traj_kernel(const
     }
     if (tid == 0 && rank == 0) {
         *ra.xs.split = sp;
-        atomicMax(ra.xs.xmax_bits, __float_as_uint(static_cast<float>(sum_s[kPartXmax])));
+        const float m = static_cast<float>(sum_s[kPartXmax]);
+        atomicMax(ra.xs.xmax_bits, __float_as_uint(isinf(m) ? sp.bound : m));
         ac.scal[kLogLik] = ll;
         ac.scal[kLogLikEnd] = ll;
         ac.scal[kSumR] = sum_r;
