@@ -81,9 +81,10 @@ def main():
     print("// largest absolute error before the coefficients' rounding: F %.1e, G %.1e." % (worst[0], worst[1]))
     print("#pragma once")
     print("constexpr int kPhiPerUnit = %d, kPhiNodes = %d, kPhiDeg = %d, kPhiRow = 10;" % (PER_UNIT, NODES, DEG))
-    print("__device__ const unsigned long long g_phi_table[kPhiNodes * kPhiRow] = {")
+    # pairs of words, so that the type carries the alignment of 16-byte loads
+    print("__device__ const ulonglong2 g_phi_table[kPhiNodes * kPhiRow / 2] = {")
     for r in rows:
-        print(",".join("0x%016xull" % v for v in r) + ",")
+        print(",".join("{0x%016xull,0x%016xull}" % (r[k], r[k + 1]) for k in range(0, len(r), 2)) + ",")
     print("};")
 
 

@@ -43,12 +43,13 @@ constexpr int kPhiBytes = kPhiNodes * kPhiRow * 8;  // 48,720
 static_assert(kPhiDeg == 5 && kPhiPerUnit == 64 && kPhiRow == 10 && kPhiBytes % 16 == 0,
               "phi_eval is written for this table");
 
+static_assert(alignof(decltype(g_phi_table)) >= 16, "phi_table_load reads it 16 bytes at a time");
+
 // The table into shared memory (16-byte aligned), by all threads of the CTA;
 // the caller synchronises.
 __device__ __forceinline__ void phi_table_load(double *tab) {
-    const ulonglong2 *src = reinterpret_cast<const ulonglong2 *>(g_phi_table);
     ulonglong2 *dst = reinterpret_cast<ulonglong2 *>(tab);
-    for (int i = threadIdx.x; i < kPhiBytes / 16; i += blockDim.x) dst[i] = src[i];
+    for (int i = threadIdx.x; i < kPhiBytes / 16; i += blockDim.x) dst[i] = g_phi_table[i];
 }
 
 // sigma in the forms the pair needs.
