@@ -310,7 +310,8 @@ int mds_far_blocks(mds_ctx *ctx, int64_t *far, int64_t *total);
 int mds_get_order(const mds_ctx *ctx, int32_t *perm);
 
 /* Cut-off z_c of the Phi-term skip of the FP32C pass: 0 turns it off, else
- * z_c >= 8 (default 8).  The FP64 path evaluates Phi for every pair.
+ * z_c >= 8 (default 8).  The FP64 path has no cut-off: the Phi terms are part
+ * of every pair in which they can change a bit of what they are added to.
  * Errors: INVALID_ARG for 0 < z < 8 or a non-finite z. */
 int mds_set_tail_cutoff(mds_ctx *ctx, double z);
 

@@ -3,14 +3,16 @@
 that the FP64 pair arithmetic needs (pair_math64.cuh),
   F(z) = phi(z) / Phi(z)   and   G(z) = log Phi(z),
 phi and Phi the standard normal density and distribution function, on the
-nodes c = i / 64, i = 0 .. 608 (z up to 9.5): degree 5 in t = z - c, |t| <= 1/128,
-each the polynomial that interpolates the function at the 6 Chebyshev points
-of its interval (computed with 40 digits).  A node is 10 words of 64 bits, low
-half first:
-  F's coefficients of t^3, t^2, t, 1 and G's of t^3, t^2, t in FP64, G's
-  constant as an integer in units of 2^-52, {F's of t^5, F's of t^4} and
-  {G's of t^5, G's of t^4} in FP32 (t^4 <= 3.7e-9: their rounding is below
-  1e-16 of the value).
+nodes c = i / 64, i = 0 .. 640 (z up to 10): degree 7 in t = z - c, |t| <= 1/128,
+each the polynomial that interpolates the function at the 8 Chebyshev points
+of its interval (computed with 60 digits).  The degree and the split of the
+coefficients keep the relative error of both functions near FP64's rounding up
+to z = 10, where they are 1e-22: a term of degree k is at most (z t)^k / k! of
+the value, so the FP32 rounding of those of degree 5 and up stays below 4e-16
+of it at z = 8 and 1.1e-15 at z = 10.  A node is 14 words of 64 bits, low half first:
+  F's coefficients of t^4, t^3, t^2, t, 1 and G's of 1 and of t^4, t^3, t^2, t
+  in FP64; in FP32 {F's of t^7, t^6}, {F's of t^5, G's of t^5}, {G's of t^7,
+  t^6}; an unused word (a row is then a whole number of 16-byte loads).
 
 Usage: python gen_phi_table.py > phi_table.h
 """
@@ -18,8 +20,8 @@ import struct
 
 from mpmath import cos, erfc, exp, log, mp, mpf, nint, pi, sqrt
 
-mp.dps = 40
-PER_UNIT, NODES, DEG = 64, 609, 5
+mp.dps = 60
+PER_UNIT, NODES, DEG = 64, 641, 7
 HALF = mpf(1) / (2 * PER_UNIT)
 
 
@@ -71,16 +73,16 @@ def main():
             for u in (-1, mpf(-7) / 10, mpf(-1) / 4, mpf(1) / 3, mpf(8) / 10, 1):
                 t = u * HALF
                 v = sum(a * t ** k for k, a in enumerate(p))
-                worst[q] = max(worst[q], abs(v - fn(c + t)))
+                worst[q] = max(worst[q], abs(v / fn(c + t) - 1))
             co.append(p)
         a, b = co
-        rows.append([f64(a[3]), f64(a[2]), f64(a[1]), f64(a[0]), f64(b[3]), f64(b[2]), f64(b[1]),
-                     int(nint(b[0] * 2 ** 52)) & (2 ** 64 - 1), f32(a[5], a[4]), f32(b[5], b[4])])
+        rows.append([f64(v) for v in (a[4], a[3], a[2], a[1], a[0], b[0], b[4], b[3], b[2], b[1])] +
+                    [f32(a[7], a[6]), f32(a[5], b[5]), f32(b[7], b[6]), 0])
     print("// Generated by gen_phi_table.py -- do not edit.")
-    print("// Node i, t = z - i/64: F = phi/Phi and G = log Phi as degree-5 polynomials (layout: see the generator);")
-    print("// largest absolute error before the coefficients' rounding: F %.1e, G %.1e." % (worst[0], worst[1]))
+    print("// Node i, t = z - i/64: F = phi/Phi and G = log Phi as degree-7 polynomials (layout: see the generator);")
+    print("// largest relative error before the coefficients' rounding: F %.1e, G %.1e." % (worst[0], worst[1]))
     print("#pragma once")
-    print("constexpr int kPhiPerUnit = %d, kPhiNodes = %d, kPhiDeg = %d, kPhiRow = 10;" % (PER_UNIT, NODES, DEG))
+    print("constexpr int kPhiPerUnit = %d, kPhiNodes = %d, kPhiDeg = %d, kPhiRow = 14;" % (PER_UNIT, NODES, DEG))
     # pairs of words, so that the type carries the alignment of 16-byte loads
     print("__device__ const ulonglong2 g_phi_table[kPhiNodes * kPhiRow / 2] = {")
     for r in rows:

@@ -76,6 +76,7 @@ __global__ void __launch_bounds__(kLpdThreads, 2)
         root64(d2, delta, inv);
         const double u = (widen(y) - delta) * sg.inv_s;
         double lp = fma(-0.5 * u, u, log_norm);
+        // beyond the table Phi is 1 - 8e-24 at least: no factor of a density
         if (phi_near(sg, delta)) lp -= phi_log(tab, sg, delta);
         if (!isfinite(lp)) atomicOr(err, kErrNonfinite);
         if (first) {

@@ -16,7 +16,7 @@
 // that of the FP64 path (pair_math64.cuh), bound by the FP64 pipe; log Phi
 // and the other scalar terms are evaluated only for j > i.  A whole CTA per
 // row rather than a warp: the rows then come in pieces small enough to end
-// together on 152 SMs.  The CTAs are resident all at once, two to four per SM,
+// together on 152 SMs.  The CTAs are resident all at once, two or three per SM,
 // and load the table once; how many, by what the last round leaves idle
 // (row_blocks): a CTA per row, left to the scheduler, took
 // 78 us at N = 600 (64), 400 at N = 2400 (351), D = 2, and 609 at N = 3001,
@@ -63,7 +63,6 @@ struct RowSums {
 template <int D, bool SCALARS>
 __device__ __forceinline__ void row_part(const double *tab, const Sigma64 &sg, const double (&xi)[D],
                                          const double *x, const float *yrow, int64_t lo, int64_t hi, RowSums<D> &acc) {
-    int64_t log_units = 0;  // at most 512 terms of at most 0.7 * 2^52
     for (int64_t j0 = lo; j0 < hi; j0 += kNaThreads) {
         const bool in = j0 + threadIdx.x < hi;
         const int64_t j = in ? j0 + threadIdx.x : lo;
@@ -85,8 +84,17 @@ __device__ __forceinline__ void row_part(const double *tab, const Sigma64 &sg, c
             phi_eval<SCALARS>(tab, sg, del, near, F, G);
             if constexpr (SCALARS) {
                 acc.v[D + 1] = fma(F, del, acc.v[D + 1]);
-                acc.v[D + 2] = fma(G.slope, G.t, acc.v[D + 2]);
-                log_units += G.units;
+                acc.v[D + 2] = fma(G.slope, G.t, acc.v[D + 2]) + G.g0;
+            }
+            w = fma(F, sg.neg_s, w);
+        }
+        const bool tiny = in && !near && phi_tiny(sg, w);
+        if (__any_sync(0xffffffffu, tiny)) {
+            double F, G;
+            phi_far<SCALARS>(sg, del, w, tiny, F, G);
+            if constexpr (SCALARS) {
+                acc.v[D + 1] = fma(F, del, acc.v[D + 1]);
+                acc.v[D + 2] += G;
             }
             w = fma(F, sg.neg_s, w);
         }
@@ -94,7 +102,6 @@ __device__ __forceinline__ void row_part(const double *tab, const Sigma64 &sg, c
 #pragma unroll
         for (int k = 0; k < D; ++k) acc.v[k] = fma(w, dl[k], acc.v[k]);
     }
-    if constexpr (SCALARS) acc.v[D + 2] = fma(static_cast<double>(log_units), kPhiUnit, acc.v[D + 2]);
 }
 
 template <int D>
@@ -154,12 +161,13 @@ __global__ void noalloc_sum_kernel(int nblocks, double *part) {
     if (threadIdx.x < 3) part[kNaMaxBlocks * kNaParts + threadIdx.x] = sm[threadIdx.x][0];
 }
 
-// CTAs for n rows: k per SM, k = 4, 3 or 2.  An SM's FP64 pipes are shared, so
-// its time is k times its largest CTA's number of rows, ceil(n / (k SMs)):
-// the k with the smallest product, more CTAs (latency) where they are equal.
+// CTAs for n rows: k per SM, k = 3 (as many as the table leaves room for) or 2.
+// An SM's FP64 pipes are shared, so its time is k times its largest CTA's
+// number of rows, ceil(n / (k SMs)): the k with the smaller product, more CTAs
+// (latency) where they are equal.
 int64_t row_blocks(int64_t n, int sms) {
     int64_t best = 0, cost = 0;
-    for (int64_t k = 4; k >= 2; --k) {
+    for (int64_t k = 3; k >= 2; --k) {
         const int64_t c = k * ((n + k * sms - 1) / (k * sms));
         if (best == 0 || c < cost) {
             best = k;

@@ -217,7 +217,7 @@ __global__ void __launch_bounds__(kPairThreads, (D <= 2 ? 4 : D <= 4 ? 3 : 2)) p
 // a time), the row block's locations and the table of phi/Phi and log Phi in
 // shared memory.  Bound by the FP64 pipe (pair_math64.cuh): per pair and
 // coordinate the difference, its square and the two accumulations (4), and
-// 11 + 11 for the rest, the latter only where some lane of the warp has z < 9.5.
+// 11 + 14 for the rest, the latter only where some lane of the warp has z <= 10.
 // The weight is summed in units of -sigma^2, so that its two terms take one
 // FMA; the partial sums carry the factor -1/sigma^2.
 template <int D>
@@ -266,7 +266,6 @@ __global__ void __launch_bounds__(kPairThreads, D <= 4 ? 3 : 2) pair_f64_kernel(
 #pragma unroll
         for (int k = 0; k < D; ++k) racc[r][k] = 0.0;
     double e2 = 0.0, md = 0.0, lp = 0.0;
-    int64_t log_units = 0;  // at most 32 pairs of each of 16 tiles, 0.7 * 2^52 each
     double *colp_base = reinterpret_cast<double *>(a.col_part);
     for (int jt = 0; jt < nst; ++jt) {
         const int J = st.j0 + jt;
@@ -316,8 +315,15 @@ __global__ void __launch_bounds__(kPairThreads, D <= 4 ? 3 : 2) pair_f64_kernel(
                         double F;
                         PhiLog G;
                         phi_eval<true>(tab, sg, del, near, F, G);
-                        lp = fma(G.slope, G.t, lp);
-                        log_units += G.units;
+                        lp = fma(G.slope, G.t, lp) + G.g0;
+                        md = fma(F, del, md);
+                        w = fma(F, sg.neg_s, w);
+                    }
+                    const bool tiny = valid && !near && phi_tiny(sg, w);
+                    if (__any_sync(0xffffffffu, tiny)) {
+                        double F, G;
+                        phi_far<true>(sg, del, w, tiny, F, G);
+                        lp += G;
                         md = fma(F, del, md);
                         w = fma(F, sg.neg_s, w);
                     }
@@ -364,7 +370,7 @@ __global__ void __launch_bounds__(kPairThreads, D <= 4 ? 3 : 2) pair_f64_kernel(
             red[(warp * kTile + 2 * (la + 8 * q) + h) * D + k] = rv[i];
         }
     }
-    double sv[3] = {e2, md, fma(static_cast<double>(log_units), kPhiUnit, lp)};
+    double sv[3] = {e2, md, lp};
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
         double v = sv[i];
