@@ -587,7 +587,8 @@ const char *mds_batch_last_error(const mds_batch *b);
  * the caller.  Nothing in it needs clearing: every slot a call reads is
  * written earlier in the same call.  The first call on each device looks up
  * the scratch's device address (cudaGetSymbolAddress) with that device
- * current and keeps it for the life of the process; make that first call
+ * current and keeps it for the life of the process, and sets the kernels'
+ * shared memory limit, for every D; make that first call
  * before any stream capture, and do not use this entry point on a device
  * after cudaDeviceReset there (the kept address would belong to the
  * destroyed context).  Each pair is

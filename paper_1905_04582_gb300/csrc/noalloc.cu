@@ -177,6 +177,23 @@ int64_t row_blocks(int64_t n, int sms) {
     return std::min<int64_t>(n, std::min<int64_t>(best * sms, kNaMaxBlocks));
 }
 
+template <int D>
+cudaError_t raise_smem_d() {
+    return cudaFuncSetAttribute(noalloc_rows_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPhiBytes);
+}
+
+// The kernels' shared memory limit, for every D at once: a later call neither
+// sets an attribute nor grows a host table.
+cudaError_t raise_smem_all() {
+    cudaError_t (*const raise[])() = {raise_smem_d<1>, raise_smem_d<2>, raise_smem_d<3>, raise_smem_d<4>,
+                                      raise_smem_d<5>, raise_smem_d<6>, raise_smem_d<7>, raise_smem_d<8>};
+    for (auto f : raise) {
+        const cudaError_t e = f();
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
 // Device address of the scratch array on the current device (looked up once
 // per device; host code cannot use the symbol itself as a device pointer).
 int scratch_address(double **out, int *sms) {
@@ -201,6 +218,11 @@ int scratch_address(double **out, int *sms) {
         e = cudaDeviceGetAttribute(&g_na_sms[dev], cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess) {
             mds::set_thread_error("mds_loglik_grad_noalloc: cudaDeviceGetAttribute: %s", cudaGetErrorString(e));
+            return MDS_ERR_CUDA;
+        }
+        e = raise_smem_all();
+        if (e != cudaSuccess) {
+            mds::set_thread_error("mds_loglik_grad_noalloc: shared memory: %s", cudaGetErrorString(e));
             return MDS_ERR_CUDA;
         }
         g_na_ptr[dev] = static_cast<double *>(p);
@@ -234,27 +256,20 @@ extern "C" int mds_loglik_grad_noalloc(int64_t n, int32_t d, const float *y, int
     if (st != MDS_OK) return st;
     const int64_t nblocks = row_blocks(n, sms);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    cudaError_t e = cudaSuccess;
     const Sigma64 sg = sigma64(sigma);
     switch (d) {
 #define MDS_NA_CASE(DD)                                                                                           \
     case DD:                                                                                                      \
-        e = mds::raise_dyn_smem(reinterpret_cast<const void *>(noalloc_rows_kernel<DD>), kPhiBytes);              \
-        if (e == cudaSuccess)                                                                                     \
-            noalloc_rows_kernel<DD>                                                                               \
-                <<<static_cast<int>(nblocks), kNaThreads, kPhiBytes, s>>>(n, y, ld, x, sg, grad, part);          \
+        noalloc_rows_kernel<DD>                                                                                   \
+            <<<static_cast<int>(nblocks), kNaThreads, kPhiBytes, s>>>(n, y, ld, x, sg, grad, part);              \
         break;
         MDS_NA_CASE(1) MDS_NA_CASE(2) MDS_NA_CASE(3) MDS_NA_CASE(4)
         MDS_NA_CASE(5) MDS_NA_CASE(6) MDS_NA_CASE(7) MDS_NA_CASE(8)
 #undef MDS_NA_CASE
         default: break;
     }
-    if (e != cudaSuccess) {
-        mds::set_thread_error("mds_loglik_grad_noalloc: shared memory: %s", cudaGetErrorString(e));
-        return MDS_ERR_CUDA;
-    }
     noalloc_sum_kernel<<<1, 256, 0, s>>>(static_cast<int>(nblocks), part);
-    e = cudaGetLastError();
+    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
         mds::set_thread_error("mds_loglik_grad_noalloc: launch: %s", cudaGetErrorString(e));
         return MDS_ERR_CUDA;
