@@ -103,9 +103,9 @@ __device__ __forceinline__ void chunk_pass(const PairArgs &a, unsigned cta) {
     extern __shared__ __align__(128) unsigned char smem_cta[];
     // group, warp within it, thread within it, and the group's chunk
     const int lane = static_cast<int>(threadIdx.x) & 31;
-    const int grp = static_cast<int>(threadIdx.x >> 5) / kPairWarps;
-    const int warp = static_cast<int>(threadIdx.x >> 5) % kPairWarps;
-    const int tid = static_cast<int>(threadIdx.x) % kPairThreads;
+    const int grp = G > 1 ? static_cast<int>(threadIdx.x >> 5) / kPairWarps : 0;
+    const int warp = static_cast<int>(threadIdx.x >> 5) - grp * kPairWarps;
+    const int tid = static_cast<int>(threadIdx.x) - grp * kPairThreads;
     const unsigned vb = cta * G + static_cast<unsigned>(grp);
     unsigned char *const smem = smem_cta + grp * align128(L::kBytes);
     pdl_trigger();
