@@ -3431,13 +3431,14 @@ int batch_check_errors(mds_batch *b, const char *what) {
 }
 
 std::mutex g_btune_mu;
-std::map<std::tuple<std::string, std::vector<int64_t>, int>, int> g_btune_cache;
+// by device, N and chains of every dataset, D, order: what the candidates and their times depend on
+std::map<std::tuple<std::string, std::vector<int64_t>, std::vector<int32_t>, int, bool>, int> g_btune_cache;
 
 // Batch strip length: forced, cached, or timed over a few candidates.
 int batch_autotune(mds_batch *b) {
     int s = b->strip_req;
     if (s == 0) {
-        const auto key = std::make_tuple(b->device_name, b->n, static_cast<int>(b->d));
+        const auto key = std::make_tuple(b->device_name, b->n, b->chains, static_cast<int>(b->d), b->ctx[0]->reordered);
         {
             std::lock_guard<std::mutex> lk(g_btune_mu);
             auto it = g_btune_cache.find(key);
