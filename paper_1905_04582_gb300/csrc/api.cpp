@@ -3303,7 +3303,8 @@ int batch_tables(mds_batch *b, int strip) {
     // the resident CTAs (see reduce_batch_kernel)
     int64_t blocks = 0;
     for (const mds_ctx *c : b->ctx) blocks += c->nt;
-    const int quarters = blocks * kReduceQuarters > static_cast<int64_t>(b->sm_count) * kReduceResident ? 1 : kReduceQuarters;
+    const int64_t resident = static_cast<int64_t>(b->sm_count) * reduce_resident(static_cast<int>(b->d));
+    const int quarters = blocks * kReduceQuarters > resident ? 1 : kReduceQuarters;
     if (quarters != b->quarters) b->gen++;
     b->quarters = quarters;
     for (int dd = 0; dd < b->n_data; ++dd) {

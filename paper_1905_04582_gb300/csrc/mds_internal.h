@@ -355,7 +355,9 @@ struct ReduceArgs {
 // The reduction runs kReduceQuarters CTAs per column block (16 items each)
 // plus one CTA for the scalars.
 constexpr int kReduceQuarters = 4;
-constexpr int kReduceResident = 4;  // CTAs per SM that the batched reduction is compiled for
+// CTAs per SM that the batched reduction is compiled for (its registers: 64 up
+// to D = 4, 80 at D = 5, 88 to 111 beyond)
+__host__ __device__ constexpr int reduce_resident(int d) { return d <= 4 ? 4 : d == 5 ? 3 : 2; }
 cudaError_t launch_reduce(const ReduceArgs &a, cudaStream_t s);
 
 // Trajectory start: (optionally) draw / load p, save x0 and the cached

@@ -495,11 +495,14 @@ __global__ void __launch_bounds__(kRedThreads) reduce_kernel(const __grid_consta
 // Batched: job (problem index, CTA of its column blocks, or -1 for the
 // scalars) per CTA.  ROWS = 64: a CTA per column block.  A CTA's time is a
 // chain of latencies (job, arguments, partials, state), so quarter blocks
-// cost when there are more of them than resident CTAs (2784 quarters on 152
-// SMs took 24 us of ncu's cold time for the 32 chains above; 728 blocks are
-// about one wave).
+// cost when there are more of them than resident CTAs (2784 CTAs for 32 chains
+// of N = 1600 to 992 took 24 us of ncu's cold time; 720 are about one wave).
+// A batched pass with its reduction, us, quarters / whole blocks: D = 6, two
+// CTAs per SM, 240 quarters 17.2 / 17.2, 320 19.5 / 17.7, 600 29.0 / 24.4;
+// D = 5, three, 440 quarters 16.1 / 16.6, 520 23.4 / 21.5; D = 8, two, 320
+// 24.9 / 22.5.
 template <int D, int ROWS>
-__global__ void __launch_bounds__(kRedThreads, D <= 4 ? kReduceResident : 2)
+__global__ void __launch_bounds__(kRedThreads, reduce_resident(D))
     reduce_batch_kernel(const ReduceArgs *cfg, const int2 *jobs, int mode) {
     const int2 job = jobs[blockIdx.x];
     reduce_body<float, D, ROWS>(cfg[job.x], mode, job.y);
