@@ -50,9 +50,13 @@ def fp32_ops_per_pair(d, far_frac=0.0, chunked=True):
     lies at z >= 8 (Phi terms skipped); with Phi: the exp argument, the Mills
     ratio P and D (3 + 3), D Phi, 1/Phi, phi/Phi, the log-product, m delta and
     one more for the weight: 8 D + 20.  The strip pass (pair_math.cuh) takes
-    8 D + 9 and 8 D + 22.  far_frac is the fraction of warp blocks that took
-    the far body."""
+    8 D + 9 and 8 D + 22.  On a line (D = 1) delta needs no root and no
+    residual: 3 fewer, 4 in the strip pass.  far_frac is the fraction of warp
+    blocks that took the far body."""
     far, near = (8 * d + 7, 8 * d + 20) if chunked else (8 * d + 9, 8 * d + 22)
+    if d == 1:
+        line = 3 if chunked else 4
+        far, near = far - line, near - line
     return (1.0 - far_frac) * near + far_frac * far
 
 

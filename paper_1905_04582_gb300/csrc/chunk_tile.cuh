@@ -22,6 +22,10 @@ __device__ __forceinline__ float half_of(float x) { return __int_as_float(__floa
 template <int D>
 __device__ __forceinline__ void geom2(const float4 (&xi)[D], const float4 (&xj)[D], float2 y2, float2 (&s)[D],
                                       float2 &d2, float2 &inv, float2 &del, float2 &e) {
+    if constexpr (D == 1) {
+        geom_line(xi[0], xj[0], y2, s[0], d2, inv, del, e);
+        return;
+    }
     float2 d2h, cr;
 #pragma unroll
     for (int k = 0; k < D; ++k) {

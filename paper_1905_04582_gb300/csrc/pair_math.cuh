@@ -176,13 +176,39 @@ __device__ __forceinline__ int reduced_base(int lane, int first_bit, bool &write
     return base;
 }
 
-// One row pair (rows r, r+1 packed) against one column: the whole per-pair
-// body of Eq. (2) and Eq. (9) for two pairs at once.
-template <int D, bool MASKED, typename K>
-__device__ __forceinline__ void pair2_f32(const K &a, const float4 (&xi)[D], const float4 (&xj)[D], float2 y2,
-                                          float2 vmask, float2 (&racc)[D], float2 (&cacc)[D], float2 &e2,
-                                          float2 &md, float2 &prod) {
-    float2 s[D];
+// Geometry of two pairs on a line (D = 1).  There delta is |x_i - x_j| itself:
+// no root, and s + r = Dh + Dl without an error, so that e = y - delta comes
+// from s and r directly.  The general form below takes d^2 as Dh^2 plus a
+// correction, which cancel where two items lie close together on the two sides
+// of a border between multiples of q: with |x_i - x_j| < 2^-12 q what is left
+// is rounding, negative half of the time.  In one dimension items come that
+// close (N = 1673 in 6 clusters: 1e-4 of the evaluations, and HMC steps ended
+// as non-finite); in two and more all their coordinates would have to (about
+// 2e-8 of the evaluations at N = 5392, D = 2).
+__device__ __forceinline__ void geom_line(const float4 &xi, const float4 &xj, float2 y2, float2 &s, float2 &d2,
+                                          float2 &inv, float2 &del, float2 &e) {
+    const float2 dh = add2(f2(xi.x, xi.y), f2(xj.x, xj.y));  // exact
+    const float2 dl = add2(f2(xi.z, xi.w), f2(xj.z, xj.w));
+    s = add2(dh, dl);
+    const float2 r = add2(add2(dh, neg2(s)), dl);  // exact: |Dh| >= |Dl| or Dh = 0
+    d2 = fma2(s, s, f2(FLT_MIN, FLT_MIN));         // FLT_MIN: see pair2_geom
+    inv = f2(rsqrt_approx(d2.x), rsqrt_approx(d2.y));
+    del = f2(fabsf(s.x), fabsf(s.y));
+    // r with the sign of s on it
+    const float2 rs = f2(__int_as_float(__float_as_int(r.x) ^ (__float_as_int(s.x) & 0x80000000)),
+                         __int_as_float(__float_as_int(r.y) ^ (__float_as_int(s.y) & 0x80000000)));
+    e = add2(add2(y2, neg2(del)), neg2(rs));
+}
+
+// The geometry of two pairs: s = x_i - x_j, d^2, 1 / delta, delta and
+// e = y - delta.
+template <int D>
+__device__ __forceinline__ void pair2_geom(const float4 (&xi)[D], const float4 (&xj)[D], float2 y2, float2 (&s)[D],
+                                           float2 &d2, float2 &inv, float2 &del, float2 &e) {
+    if constexpr (D == 1) {
+        geom_line(xi[0], xj[0], y2, s[0], d2, inv, del, e);
+        return;
+    }
     float2 d2h, cr;
 #pragma unroll
     for (int k = 0; k < D; ++k) {
@@ -199,14 +225,24 @@ __device__ __forceinline__ void pair2_f32(const K &a, const float4 (&xi)[D], con
     }
     // d^2 = d2h + cr (+FLT_MIN keeps rsqrt finite for coincident points, whose
     // delta is then ~1e-19 and whose gradient term is exactly 0)
-    const float2 d2 = add2(d2h, cr);
-    const float2 inv = f2(rsqrt_approx(d2.x), rsqrt_approx(d2.y));
-    const float2 del = f2(sqrt_approx(d2.x), sqrt_approx(d2.y));  // MUFU, frees an FMA-pipe slot
+    d2 = add2(d2h, cr);
+    inv = f2(rsqrt_approx(d2.x), rsqrt_approx(d2.y));
+    del = f2(sqrt_approx(d2.x), sqrt_approx(d2.y));  // MUFU, frees an FMA-pipe slot
     // residual of the square root: true d^2 - del^2 = (d2h - del^2) + cr;
     // delta_true = del + res / (2 del) to first order
     const float2 res = add2(fma2(neg2(del), del, d2h), cr);
     const float2 hinv = mul2(inv, f2(0.5f, 0.5f));
-    float2 e = fma2(neg2(res), hinv, add2(y2, neg2(del)));        // y - delta, corrected
+    e = fma2(neg2(res), hinv, add2(y2, neg2(del)));        // y - delta, corrected
+}
+
+// One row pair (rows r, r+1 packed) against one column: the whole per-pair
+// body of Eq. (2) and Eq. (9) for two pairs at once.
+template <int D, bool MASKED, typename K>
+__device__ __forceinline__ void pair2_f32(const K &a, const float4 (&xi)[D], const float4 (&xj)[D], float2 y2,
+                                          float2 vmask, float2 (&racc)[D], float2 (&cacc)[D], float2 &e2,
+                                          float2 &md, float2 &prod) {
+    float2 s[D], d2, inv, del, e;
+    pair2_geom<D>(xi, xj, y2, s, d2, inv, del, e);
     // Phi via the Mills ratio: phi' = exp(-z^2/2), -P/sqrt(2 pi) and D in delta
     const float2 ea = mul2(d2, a.c_phi);
     const float2 ph = f2(ex2_approx(ea.x), ex2_approx(ea.y));
@@ -247,27 +283,8 @@ __device__ __forceinline__ void pair2_f32(const K &a, const float4 (&xi)[D], con
 template <int D, typename K>
 __device__ __forceinline__ void pair2_far(const K &a, const float4 (&xi)[D], const float4 (&xj)[D], float2 y2,
                                           float2 (&racc)[D], float2 (&cacc)[D], float2 &e2) {
-    float2 s[D];
-    float2 d2h, cr;
-#pragma unroll
-    for (int k = 0; k < D; ++k) {
-        const float2 dh = add2(f2(xi[k].x, xi[k].y), f2(xj[k].x, xj[k].y));
-        const float2 dl = add2(f2(xi[k].z, xi[k].w), f2(xj[k].z, xj[k].w));
-        s[k] = add2(dh, dl);
-        if (k == 0) {
-            d2h = mul2(dh, dh);
-            cr = fma2(dl, add2(s[k], dh), f2(FLT_MIN, FLT_MIN));
-        } else {
-            d2h = fma2(dh, dh, d2h);
-            cr = fma2(dl, add2(s[k], dh), cr);
-        }
-    }
-    const float2 d2 = add2(d2h, cr);
-    const float2 inv = f2(rsqrt_approx(d2.x), rsqrt_approx(d2.y));
-    const float2 del = f2(sqrt_approx(d2.x), sqrt_approx(d2.y));
-    const float2 res = add2(fma2(neg2(del), del, d2h), cr);
-    const float2 hinv = mul2(inv, f2(0.5f, 0.5f));
-    const float2 e = fma2(neg2(res), hinv, add2(y2, neg2(del)));
+    float2 s[D], d2, inv, del, e;
+    pair2_geom<D>(xi, xj, y2, s, d2, inv, del, e);
     e2 = fma2(e, e, e2);
     // w / delta = -(y - delta) / (sigma^2 delta)
     const float2 wi = mul2(mul2(e, a.neg_inv_s2), inv);
