@@ -386,7 +386,7 @@ def batch_entry(reps, steps):
         mc.set_sigma(ds[0].sigma)
         ceil_near = mc.pair_body_ceiling(far=False)
     shape = (f"batched strip kernel, {strip} tiles per strip" if strip > 0 else
-             f"every chain's chunked pass (about {-strip} tiles per chunk) as concurrent graph branches")
+             f"every chain's chunked pass (about {-strip} tiles per chunk) in one launch")
     return {"datasets": [w.n for w in ds], "chains_per_dataset": chains, "order": "locality (mds_batch_reorder)",
             "strip": strip,
             "shape": shape,

@@ -46,11 +46,11 @@ __global__ void ho_restore_kernel(float *y, const int64_t *off, int64_t count, c
 // lp = log p(y | delta, sigma) of every held-out pair.  Bound by the FP64 pipe
 // like the FP64 pair pass, so it takes that pass's forms (pair_math64.cuh):
 // delta without a square root, log Phi from the table, the constants of sigma
-// from the host; about 24 FP64 instructions a pair at D = 3 where CUDA's
+// from the host; about 26 FP64 instructions a pair at D = 3 where CUDA's
 // sqrt, divisions, erfc and log1p took about 220.  Two CTAs per SM, each with
-// the table in shared memory, the pairs in turn.  Measured (GB300, the
-// whole fold: gradient, one draw, sum): N = 2999, D = 3, 225,000 held-out
-// pairs 220 -> 156 us.
+// the table in shared memory and a contiguous share of the pairs.  Measured
+// (GB300, the whole fold: gradient, one draw, sum): N = 2999, D = 3, 225,000
+// held-out pairs 221 -> 104 us, the waits and the sum's one launch included.
 template <typename T>
 __global__ void __launch_bounds__(kLpdThreads, 2)
     lpd_accumulate_kernel(const T *x, int d, const int2 *pairs, const float *ho_y, int64_t count, Sigma64 sg,

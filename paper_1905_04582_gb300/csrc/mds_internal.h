@@ -110,7 +110,7 @@ enum ScalarPart : int {
 // Dh = xh_i - xh_j and Dh^2 are exact in FP32, sum_k Dh_k^2 is exact, and
 // the squared distance is sum_k Dh^2 + Dl (2 Dh + Dl) with Dl = xl_i - xl_j,
 // a small correction computed in FP32 -- which keeps y - delta accurate where
-// y and delta nearly cancel.
+// y and delta nearly cancel.  (D = 1: delta is |x_i - x_j|, geom_line.)
 //   xrow[(I * D + k) * 32 + r] (float4) = { xh_{i,k}, xh_{i+1,k}, xl_{i,k}, xl_{i+1,k} },
 //        i = 64 I + 2 r (row block I, row pair r: D x 32 float4, contiguous)
 //   xcol[(j  * D + k)] (float4) = { -xh_{j,k}, -xh_{j,k}, -xl_{j,k}, -xl_{j,k} }

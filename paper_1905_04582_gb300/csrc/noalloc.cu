@@ -18,11 +18,11 @@
 // row rather than a warp: the rows then come in pieces small enough to end
 // together on 152 SMs.  The CTAs are resident all at once, two or three per SM,
 // and load the table once; how many, by what the last round leaves idle
-// (row_blocks): a CTA per row, left to the scheduler, took
-// 78 us at N = 600 (64), 400 at N = 2400 (351), D = 2, and 609 at N = 3001,
-// D = 3 (573, the shorter table included).  Each block writes its partial sums of the scalar
-// terms into the scratch array; a second, single-block kernel sums them in a
-// fixed order.
+// (row_blocks): at D = 2 two and three per SM take 354 and 367 us at N = 2400,
+// 955 and 925 at N = 4000.  (With a shorter table, a CTA per row left to the
+// scheduler took 400 us at N = 2400 against 351 for resident ones.)  Each
+// block writes its partial sums of the scalar terms into the scratch array; a
+// second, single-block kernel sums them in a fixed order.
 #include <cuda_runtime.h>
 
 #include <algorithm>
